@@ -580,6 +580,7 @@ extern "C" eprop_status eprop_create_network(const eprop_config *cfg, const epro
         }
         eprop::prepare_kernel_attributes();
         eprop::prepare_step_kernel_attributes();
+        eprop::prepare_sample_attributes();
         eprop::prepare_learning_signal_attributes();
         cudaError_t e = cudaDeviceSynchronize();
         if (e != cudaSuccess) { s = cuda_fail(nullptr, e, "network set-up"); goto fail_out; }
@@ -797,7 +798,11 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
         cudaEventRecord(net->ev_join, net->st2);
         cudaStreamWaitEvent(st, net->ev_join, 0);
     };
-    const bool persistent = c.launch_mode == 2;
+    // small networks run the steps of a window sample by sample in one launch
+    // (every launch mode); larger ones with launch_mode 2 run all steps of the
+    // call in one cooperative launch, else a few launches per step
+    const bool sample_loop = eprop::sample_steps_fit(n);
+    const bool persistent = c.launch_mode == 2 && !sample_loop;
     if (persistent) {
         // form (2): every step of the call in one cooperative launch
         cudaError_t le = eprop::launch_persistent_steps(n, T, net->gridbar, net->pers_blocks, st);
@@ -805,7 +810,11 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
         L += 1;
     }
     for (int i = 1; i <= T; ++i) {
-        if (persistent) {
+        if (sample_loop && (i - 1) % U == 0) {
+            eprop::launch_sample_steps(n, i, i + U - 1, st);
+            L += 1;
+        }
+        if (persistent || sample_loop) {
             if (i % U != 0) continue;
         } else {
         if (c.n_in > 0) { eprop::launch_inject(n, i, (int)net->max_in_per_step, st); L += 1; }
@@ -826,7 +835,7 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
         L += 3;
         }
         if (i % U == 0) {
-            join_readout();
+            if (!sample_loop) join_readout();    // nothing forked since the last join otherwise
             eprop::launch_filter_error(n, i, st);
             // L[b][u][j] = sum_k B[j][k] E[b][u][k] of the whole window
             // (Eq. final-gradient), tensor cores with split TF32 operands

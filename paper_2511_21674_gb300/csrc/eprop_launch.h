@@ -38,6 +38,11 @@ void launch_unpack_raster(const Net &n, unsigned char *dst, cudaStream_t st);
 void launch_adam(const Net &n, int sm_count, cudaStream_t st);
 int persistent_blocks(int sm_count);
 cudaError_t launch_persistent_steps(const Net &n, int T, GridBar *gb, int blocks, cudaStream_t st);
+// sample-resident step loop of small networks: call steps i0..i1 (one update
+// window) of every sample in one launch
+bool sample_steps_fit(const Net &n);
+void launch_sample_steps(const Net &n, int i0, int i1, cudaStream_t st);
+void prepare_sample_attributes();
 void prepare_learning_signal_attributes();
 // band-major learning state (trace_kernel 4)
 int band_width(bool alif);

@@ -5,6 +5,7 @@
 #include "eprop.h"
 #include "eprop_internal.cuh"
 #include "eprop_launch.h"
+#include "neuron_core.cuh"
 
 namespace eprop {
 
@@ -43,98 +44,35 @@ __global__ void inject_kernel(Net n, int i) {
         mark_spike(n, b, n.x_ids[q], r);
 }
 
-// One neuron's update at call step i from its loaded state (Eq. lif_update,
-// Eq. binary-spike-state-variable, Eq. spike-threshold-adaptation, the
-// surrogate): clears its ring slot, writes v, a, ref, z_prev, psi and the
-// rate regularisation signal, and marks a spike.  Shared by the per-step
-// neuron kernel and the persistent step loop.
-// VAR: the e-prop+ variants (fixed reset, ignore-and-fire, exponential
-// surrogate, rate regularisation) are compiled in; the plain method's
-// instance carries none of their code.
+// One neuron's update at call step i from its loaded state (neuron_core):
+// clears its ring slot, writes v, a, ref, z_prev, psi and the rate
+// regularisation signal, and marks a spike.  Shared by the per-step neuron
+// kernel and the persistent step loop.
 template <bool VAR>
 __device__ __forceinline__ void neuron_update(const Net &n, int i, int b, int j, long long nb, int r, int a0,
                                               long long t_abs, const uint32_t *thr_s, float *psi_row,
                                               long long *ring_row, long long acc_q, float v_hi_q, float v_lo_q,
                                               float a_hi_q, float a_lo_q, int ref_q, uint8_t zp8_q) {
     ring_row[j] = 0;
-    // exact fixed-point input split into an FP32 pair
-    const float acc_hi = (float)acc_q;
-    float u_hi = acc_hi * kFixInv;
-    float u_lo = (float)(acc_q - (long long)acc_hi) * kFixInv;
-    if (n.n_thr > 0) {
-        const uint64_t h = mix64(mix64(mix64(n.drive_seed ^ (uint64_t)j) ^ (uint64_t)t_abs) ^ (uint64_t)b);
-        const uint32_t u = (uint32_t)(h >> 32);
-        // thresholds are non-decreasing (checked at creation): the count of
-        // thresholds <= u is the index of the first one above u
-        int cnt = 0;
-        while (cnt < n.n_thr && u >= thr_s[cnt]) ++cnt;
-        const float dv = n.drive_weight * (float)cnt;
-        const float de = fmaf(n.drive_weight, (float)cnt, -dv);
-        float e;
-        two_sum(u_hi, dv, u_hi, e);
-        u_lo += e + de;
-    }
-    const float zp = (float)zp8_q;
-    float vth = n.v_th, vth_lo = 0.0f;
-    if (n.alif) {
-        comp_step(n.rho, n.rho_lo, zp, 0.0f, a_hi_q, a_lo_q);
-        n.a[nb] = a_hi_q;
-        n.a_lo[nb] = a_lo_q;
-        vth = fmaf(n.beta_a, a_hi_q, n.v_th);
-        vth_lo = fmaf(n.beta_a, a_hi_q, n.v_th - vth) + n.beta_a * a_lo_q;
-    }
-    if (VAR && n.reset_mode == 1 && zp != 0.0f) {
-        // fixed reset: v' = v_reset + I (the decayed membrane is replaced)
-        float s, e;
-        two_sum(n.v_reset, u_hi, s, e);
-        const float lo = e + u_lo;
-        const float hi = s + lo;
-        v_lo_q = lo - (hi - s);
-        v_hi_q = hi;
-    } else {
-        // v' = alpha v + I - z_prev v_th (Eq. lif_update), input term as a pair
-        if (!VAR || n.reset_mode == 0) {
-            float e;
-            two_sum(u_hi, -zp * vth, u_hi, e);
-            u_lo += e - zp * vth_lo;
-        }
-        comp_step(n.alpha, n.alpha_lo, u_hi, u_lo, v_hi_q, v_lo_q);
-    }
-    n.v[nb] = v_hi_q;
-    n.v_lo[nb] = v_lo_q;
-    const float m = (v_hi_q - vth) + (v_lo_q - vth_lo);
-    const bool refractory = ref_q > 0;
-    int z;
-    if (n.forced) {
-        z = n.forced[((long long)b * n.T + (i - 1)) * n.n_rec + j] ? 1 : 0;
-    } else if (VAR && n.if_period > 0) {
-        // ignore-and-fire: a fixed schedule with the neuron's own phase
-        const uint32_t ph = (uint32_t)(mix64(n.if_seed ^ (uint64_t)j) >> 32) % (uint32_t)n.if_period;
-        z = ((t_abs + (long long)ph) % n.if_period) == 0 ? 1 : 0;
-    } else {
-        z = (!refractory && m > 0.0f) ? 1 : 0;
-    }
+    NeuronRegs s{v_hi_q, v_lo_q, a_hi_q, a_lo_q, ref_q, (float)zp8_q, 0.0f};
+    if (VAR && n.R_win) s.rate = n.rate[nb];
+    const int forced_z = n.forced ? (n.forced[((long long)b * n.T + (i - 1)) * n.n_rec + j] ? 1 : 0) : -1;
     float psi;
-    if (VAR && n.surrogate == 1) {      // Eq. exponential-surrogate-gradient
-        psi = refractory ? 0.0f : n.gamma * expf(-n.beta_sg * fabsf(m));
-    } else {                     // Eq. piecewise-linear-surrogate-gradient
-        const float hh = 1.0f - n.beta_sg * fabsf(m);
-        psi = refractory ? 0.0f : n.gamma * fmaxf(hh, 0.0f);
+    int z;
+    neuron_core<VAR>(n, b, j, t_abs, thr_s, acc_q, forced_z, s, psi, z);
+    if (n.alif) {
+        n.a[nb] = s.a_hi;
+        n.a_lo[nb] = s.a_lo;
     }
+    n.v[nb] = s.v_hi;
+    n.v_lo[nb] = s.v_lo;
     psi_row[j] = psi;
     if (VAR && n.R_win) {
-        // moving-average rate (Eq. ema-rate) and the regularisation
-        // signal of Eq. ema-gradient, with G_beta's factor (1 - beta)
-        const float f = n.beta_reg * n.rate[nb] + (1.0f - n.beta_reg) * (float)z;
-        n.rate[nb] = f;
-        n.R_win[((long long)b * n.U + (r - a0 - 1)) * n.n_rec + j] =
-            n.c_reg * (1.0f - n.beta_reg) * (f - n.f_target);
+        n.rate[nb] = s.rate;
+        n.R_win[((long long)b * n.U + (r - a0 - 1)) * n.n_rec + j] = rate_signal(n, s.rate);
     }
     if (n.record_psi) n.rec_psi[((long long)b * n.T + (i - 1)) * n.n_rec + j] = psi;
-    int rf = ref_q;
-    if (refractory) rf -= 1;
-    if (z) rf = n.t_ref;
-    n.ref[nb] = rf;
+    n.ref[nb] = s.ref;
     n.z_prev[nb] = (uint8_t)z;
     if (z) {
         mark_spike(n, b, n.n_in + j, r);
@@ -271,29 +209,16 @@ __device__ void readout_finish(const Net &n, int i, int b) {
     if (has_k) {
         const long long acc = __ldcg(n.y_acc + bk);     // summed by atomics in L2
         n.y_acc[bk] = 0;
-        y = n.kappa * n.y[bk] + (float)acc * kFixInv;
+        y = readout_step(n, n.y[bk], acc);
         n.y[bk] = y;
         n.y_rec[((long long)b * n.T + (i - 1)) * n.n_out + k] = y;
     }
     const float win = n.window ? (float)n.window[(long long)b * n.T + (i - 1)] : 1.0f;
     const float tgt = has_k ? n.targets[((long long)b * n.T + (i - 1)) * n.n_out + k] : 0.0f;
-    float l;
-    if (n.loss == 0) {
-        const float diff = y - tgt;
-        if (has_k) E[k] = win * diff;
-        l = has_k ? 0.5f * win * diff * diff : 0.0f;
-    } else if (n.loss == 2) {        // temporal MSE (Eq. temporal-mse)
-        const float diff = y - tgt;
-        const float invK = 1.0f / (float)n.n_out;
-        if (has_k) E[k] = win * (2.0f * invK) * diff;
-        l = has_k ? win * diff * diff * invK : 0.0f;
-    } else {
-        const float mx = block_max(has_k ? y : -INFINITY, sh);
-        const float ex = has_k ? expf(y - mx) : 0.0f;
-        const float den = block_sum(ex, sh);
-        if (has_k) E[k] = win * (ex / den - tgt);
-        l = has_k ? -win * tgt * ((y - mx) - logf(den)) : 0.0f;
-    }
+    float Ek;
+    const float l = error_signal(n, y, tgt, win, has_k, Ek, [&](float x) { return block_max(x, sh); },
+                                 [&](float x) { return block_sum(x, sh); });
+    if (has_k) E[k] = Ek;
     const float tot = block_sum(l, sh);
     if (threadIdx.x == 0) n.loss_acc[b] += tot;
 }
