@@ -150,7 +150,8 @@ typedef struct eprop_config {
                                  update_interval = 0), n_out <= 256 and no
                                  predictor; results are bit-identical to 0/1 */
     int32_t trace_kernel;     /* synapse-trace kernel: 0 auto (3 when state is
-                                 carried, else 2 for batch > 1, else 1);
+                                 carried, else 2 for batch > 1 or a small network
+                                 (n_rec <= 1024, <= 2^21 synapses), else 1);
                                  1 lazy window work queue (batch 1): only
                                  synapses with an arrival are touched, a
                                  skipped window is caught up at the next

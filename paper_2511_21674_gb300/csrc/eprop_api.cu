@@ -160,14 +160,13 @@ static eprop_status alloc_window(eprop_net *net, int U, int T) {
     n.kappaeU = (float)(c.kappa_e < 0.f ? std::exp(-(double)c.dt / c.tau_out * U)
                                         : std::pow((double)c.kappa_e, (double)U));
     n.RW = next_pow2((U + D + 31) / 32);
-    net->qp_stride = c.neuron_model == 1 ? 4 : 2;
-    const double qp_bytes = (double)U * N * net->qp_stride * 4.0 * B;
+    // window tables: (Q, Pe[, Pa]) with carried state, Q alone without
+    net->qp_stride = !n.has_state ? 1 : c.neuron_model == 1 ? 4 : 2;
     if (c.trace_kernel == 1) net->trace_mode = 0;
     else if (c.trace_kernel == 2) net->trace_mode = 1;
     else if (c.trace_kernel == 3) net->trace_mode = 2;
     else if (c.trace_kernel == 4) net->trace_mode = 3;
-    else net->trace_mode = n.has_state ? 2 : (B > 1 ? 1 : 0);
-    (void)qp_bytes;
+    else net->trace_mode = n.has_state ? 2 : (B > 1 || eprop::sample_net_small(n)) ? 1 : 0;
     // row records keep spike steps as 16-bit offsets inside the window
     if (net->trace_mode == 3 && U + D > 65536)
         return fail(net, EPROP_EINVAL, "trace_kernel 4 needs update windows of at most 65536 - max_delay steps");

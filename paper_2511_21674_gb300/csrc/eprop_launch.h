@@ -40,7 +40,8 @@ int persistent_blocks(int sm_count);
 cudaError_t launch_persistent_steps(const Net &n, int T, GridBar *gb, int blocks, cudaStream_t st);
 // sample-resident step loop of small networks: call steps i0..i1 (one update
 // window) of every sample in one launch
-bool sample_steps_fit(const Net &n);
+bool sample_net_small(const Net &n);     // sizes only
+bool sample_steps_fit(const Net &n);     // and the forms the loop serves
 void launch_sample_steps(const Net &n, int i0, int i1, cudaStream_t st);
 void prepare_sample_attributes();
 void prepare_learning_signal_attributes();

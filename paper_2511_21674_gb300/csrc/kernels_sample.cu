@@ -415,12 +415,14 @@ __global__ void __launch_bounds__(BT, 1) sample_steps_kernel(Net n, int i0, int 
     if (lists && tid < kBkt) n.list_cnt[list_index(n, b, (ck.r_base + i1 + 1) % n.RS) + tid] = 0;
 }
 
-// The loop serves the plain forms of small networks: one thread per neuron
-// (at most four), synapses that fit one SM's L1/L2 share and whose per-step
-// events one SM can add faster than a step's launches take.
+// One thread per neuron (at most four), synapses that fit one SM's L1/L2
+// share and whose per-step events one SM adds faster than a step's launches
+// take.
+bool sample_net_small(const Net &n) {
+    return n.n_rec <= kSmpMaxRec && n.n_in <= kSmpMaxIn && n.n_out <= kSmpMaxOut && n.nnz <= kSmpMaxNnz;
+}
 bool sample_steps_fit(const Net &n) {
-    return n.n_rec <= kSmpMaxRec && n.n_in <= kSmpMaxIn && n.n_out <= kSmpMaxOut && n.nnz <= kSmpMaxNnz &&
-           n.pred_mode == 0 && n.d_out == 0 && !n.band && !(n.has_state && !n.dense);
+    return sample_net_small(n) && n.pred_mode == 0 && n.d_out == 0 && !n.band && !(n.has_state && !n.dense);
 }
 
 #define EPROP_SMP_EACH(X) \

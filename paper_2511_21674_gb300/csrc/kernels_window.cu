@@ -95,14 +95,21 @@ __global__ void filter_error_kernel(Net n) {
 // the whole window beforehand on the tensor cores, L_win) are
 // loaded into registers, then the adjoint recursion writes the per-step
 // tables and, at the window start, the window coefficients.
-template <bool ALIF, bool REG, bool F64>
+// STATE: the window's end state and coefficients are wanted (carried traces).
+// Without carried state nothing reads them: only Q is swept and written, one
+// float per step and neuron.
+// The FP64 sweep is bound by an SM's FP64 pipe (2 lanes per clock: a warp
+// instruction takes 16 cycles), so the host deals it in blocks of one warp
+// until every SM has several: 100 neurons x 1000 steps 1226 us
+// in one block of four warps, 736 us in four blocks.
+template <bool ALIF, bool REG, bool F64, bool STATE>
 __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
     constexpr int kTC = ALIF ? 16 : 32;     // window steps per chunk
     const int b = blockIdx.y;
     const int U = n.U, N = n.n_rec;
     const int r_end = run_step_w(n, i_end);
     const int a0 = r_end - U;
-    const int j = blockIdx.x * 128 + threadIdx.x;
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const bool act = j < N;
     const float *psi_g = n.psi_hist + (long long)b * (U + 1) * N + (act ? j : 0);
     const float *L_g = n.L_win + (long long)b * U * N + (act ? j : 0);    // [U][N], row u - 1 = step u
@@ -177,25 +184,31 @@ __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
                     R na = g2 * ma - beta * pn * g2 * D;
                     R ne = ke * me;
                     mz = nz; ma = na; me = ne;
-                    nz = alpha * ez + p * ea + pn * g1 * ee;
-                    na = g2 * ea - beta * pn * g2 * ee;
-                    ne = ke * ee;
-                    ez = nz; ea = na; ee = ne;
-                    nz = alpha * az + p * aa + pn * g1 * ae;
-                    na = g2 * aa - beta * pn * g2 * ae;
-                    ne = ke * ae;
-                    az = nz; aa = na; ae = ne;
+                    if (STATE) {
+                        nz = alpha * ez + p * ea + pn * g1 * ee;
+                        na = g2 * ea - beta * pn * g2 * ee;
+                        ne = ke * ee;
+                        ez = nz; ea = na; ee = ne;
+                        nz = alpha * az + p * aa + pn * g1 * ae;
+                        na = g2 * aa - beta * pn * g2 * ae;
+                        ne = ke * ae;
+                        az = nz; aa = na; ae = ne;
+                    }
                 } else {
                     mz = alpha * mz + alpha * pn * D;
                     me = ke * me;
-                    ez = alpha * ez + alpha * pn * ee;
-                    ee = ke * ee;
+                    if (STATE) {
+                        ez = alpha * ez + alpha * pn * ee;
+                        ee = ke * ee;
+                    }
                 }
             }
             me += (R)Lc[c];
             if (REG) mb += (R)Rc[c];
             const R De = REG ? me + mb : me;           // adjoint of e^u
-            if (ALIF) {
+            if (!STATE) {
+                n.qp[qbase + (long long)(u - 1) * N] = (float)(mz + p * De);
+            } else if (ALIF) {
                 reinterpret_cast<float4 *>(n.qp)[qbase + (long long)(u - 1) * N] =
                     make_float4((float)(mz + p * De), (float)(ez + p * ee), (float)(az + p * ae), 0.f);
             } else {
@@ -204,7 +217,7 @@ __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
             }
             pn = p;
         }
-        if (u0 == 1) {
+        if (STATE && u0 == 1) {
             // step a0 (u = 0): the window coefficients c = (A^{a0+1})^T mu^{a0+1}
             // (regularisation runs without carried state: no coefficients
             // of F_beta are kept, only G's adjoint sees it)
@@ -235,7 +248,7 @@ __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
     if (!act) return;
     // window coefficients: c = (mz, ma, me), Phi rows (ez, ea, .) and (az, aa, .);
     // one set per sample ([B][N][RC])
-    if (n.has_state) {
+    if (STATE) {
         const int slot = (a0 / U) & (n.RC - 1);
         const long long cj = ((long long)b * N + j) * n.RC + slot;
         if (ALIF) {
@@ -300,7 +313,7 @@ __device__ __noinline__ float catch_up(const Net n, int j, int k0, int kW, float
     return G;
 }
 
-template <bool ALIF>
+template <bool ALIF, bool STATE = true>
 __device__ __noinline__ void scan_arrivals(const Net n, const uint32_t *words, int lo, int hi, int d,
                                            long long qrow, float &G, float &ebar, float &epsa) {
     const int N = n.n_rec;
@@ -315,7 +328,9 @@ __device__ __noinline__ void scan_arrivals(const Net n, const uint32_t *words, i
         while (m) {
             const int a = r + __ffs(m) - 1 + d;
             m &= m - 1;
-            if (ALIF) {
+            if (!STATE) {
+                G += n.qp[qrow + (long long)a * N];
+            } else if (ALIF) {
                 const float4 t = reinterpret_cast<const float4 *>(n.qp)[qrow + (long long)a * N];
                 G += t.x; ebar += t.y; epsa += t.z;
             } else {
@@ -535,7 +550,8 @@ __global__ void __launch_bounds__(256, 2) trace_window_kernel(Net n, int i_end) 
                 t0[u] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (has && listed) {
                     const long long qi = qa + (long long)(sp[cc] + dl) * N + j;
-                    if (ALIF) t0[u] = __ldg(reinterpret_cast<const float4 *>(n.qp) + qi);
+                    if (!STATE) t0[u].x = __ldg(n.qp + qi);
+                    else if (ALIF) t0[u] = __ldg(reinterpret_cast<const float4 *>(n.qp) + qi);
                     else {
                         const float2 t = __ldg(reinterpret_cast<const float2 *>(n.qp) + qi);
                         t0[u] = make_float4(t.x, t.y, 0.f, 0.f);
@@ -582,7 +598,9 @@ __global__ void __launch_bounds__(256, 2) trace_window_kernel(Net n, int i_end) 
                     for (int cc = c0[u] + 1; cc < ns; ++cc) {
                         const int a = sp[cc] + dl;
                         if (a > r_end) break;
-                        if (ALIF) {
+                        if (!STATE) {
+                            G += __ldg(n.qp + qa + (long long)a * N + j);
+                        } else if (ALIF) {
                             const float4 t = __ldg(reinterpret_cast<const float4 *>(n.qp) + qa + (long long)a * N + j);
                             G += t.x; ebar += t.y; epsa += t.z;
                         } else {
@@ -591,7 +609,7 @@ __global__ void __launch_bounds__(256, 2) trace_window_kernel(Net n, int i_end) 
                         }
                     }
                 } else {            // rows with more spikes than the cache holds
-                    scan_arrivals<ALIF>(n, words, max(s, a0 + 1 - dl), r_end - dl, dl, qa + j, G, ebar, epsa);
+                    scan_arrivals<ALIF, STATE>(n, words, max(s, a0 + 1 - dl), r_end - dl, dl, qa + j, G, ebar, epsa);
                 }
                 {
                     const float wn = window_update(n, q, wv[u], G);
@@ -963,63 +981,126 @@ __global__ void __launch_bounds__(256, MODE == kPassIdle ? 3 : 2) window_pass_ke
 }
 
 // event-driven synapse gradient, batched single-window form (no carried
-// state: each arrival contributes Q(a) independently).  One warp per source
-// row; the row's spikes of every sample are gathered into shared memory and
-// every synapse sums the table entries of its arrivals over all samples.
-template <int QP_STRIDE>
-__global__ void __launch_bounds__(256) trace_batched_kernel(Net n) {
-    constexpr int CAP = 512;
-    __shared__ int sp[8][CAP];      // (sample << 20) | step
-    __shared__ int ncount[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gw = blockIdx.x * (blockDim.x >> 5) + warp;
-    const int nw = gridDim.x * (blockDim.x >> 5);
+// state: each arrival contributes Q(a) independently).  One block per source
+// row: its threads scan the row's spike bits of every sample and compact them
+// (block scan, so in sample and step order) into a list in shared memory;
+// then each thread owns one synapse (or, on short rows, a share of its
+// spikes) and sums the table entries of the arrivals.  The sum (up to
+// hundreds of terms) is carried as an FP32 pair with an error-free addition
+// (TwoSum): about 48 bits for 7 FP32 operations, where an FP64 sum costs a
+// conversion and an addition of 16 cycles per warp each (2 FP64 lanes per
+// SM).  Lanes of a warp read consecutive targets of one (sample, step).
+// Measured (batch 64, 2512 rows, 5e7 arrivals): one warp per row with FP64
+// sums and a four-float table 705 us; this form 94 us; batch 32 of 2200
+// steps, 140 rows: 2063 -> 74 us.
+constexpr int kTbThreads = 256;
+constexpr int kTbCap = 32 * kTbThreads;          // spikes listed: at least one round of words
+__global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n) {
+    __shared__ int sp[kTbCap];                   // (sample << 20) | step
+    __shared__ int wsum[kTbThreads / 32];
+    __shared__ float2 red[kTbThreads];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int U = n.U, N = n.n_rec, T = n.T;
-    for (int src = gw; src < n.n_src; src += nw) {
-        const long long q0 = n.row_ptr[src], q1 = n.row_ptr[src + 1];
-        if (q1 == q0) continue;
-        // gather (sample, step) pairs; lanes split the samples
-        if (lane == 0) ncount[warp] = 0;
-        __syncwarp();
-        for (int b = lane; b < n.B; b += 32) {
-            const uint32_t *words = src_words_c(n, b, src);
-            for_each_spike(words, n.RW, 1, T, [&](int st) {
-                const int pos = atomicAdd(&ncount[warp], 1);
-                if (pos < CAP) sp[warp][pos] = (b << 20) | st;
-            });
-        }
-        __syncwarp();
-        const int ns = ncount[warp];
-        if (ns == 0) continue;
-        for (long long q = q0 + lane; q < q1; q += 32) {
-            const uint32_t td = n.tgt_d[q];
-            const int j = (int)(td & 0xFFFFFFu);
-            const int d = (int)(td >> 24);
-            // the batch's sum of arrival terms (up to samples x arrivals of
-            // them) is reduced in FP64
-            double G = 0.0;
-            if (ns <= CAP) {
-                for (int c = 0; c < ns; ++c) {
-                    const int v = sp[warp][c];
-                    const int b = v >> 20, a = (v & 0xFFFFF) + d;
-                    if (a <= T) G += (double)n.qp[(((long long)b * U + (a - 1)) * N + j) * QP_STRIDE];
+    const int wps = T / 32 + 1;                  // words per sample holding steps 1..T
+    const int nwords = n.B * wps;
+    for (int src = blockIdx.x; src < n.n_src; src += gridDim.x) {
+        const long long q0 = n.row_ptr[src];
+        const int len = (int)(n.row_ptr[src + 1] - q0);
+        if (len == 0) continue;
+        // lists the spikes of words w0.. until the list is full; returns the
+        // next word
+        int ns = 0;
+        auto fill = [&](int w0) -> int {
+            ns = 0;
+            while (w0 < nwords) {
+                const int w = w0 + tid;
+                uint32_t m = 0u;
+                int b = 0, k = 0;
+                if (w < nwords) {
+                    b = w / wps;
+                    k = w - b * wps;
+                    m = n.bits[((long long)b * n.n_src + src) * n.RW + k];
+                    if (k == 0) m &= ~1u;                                  // steps start at 1
+                    if (k == wps - 1 && (T & 31) != 31) m &= (2u << (T & 31)) - 1u;
                 }
-            } else {
-                for (int b = 0; b < n.B; ++b) {
-                    const uint32_t *words = src_words_c(n, b, src);
-                    for_each_spike(words, n.RW, 1, T - d, [&](int st) {
-                        G += (double)n.qp[(((long long)b * U + (st + d - 1)) * N + j) * QP_STRIDE];
-                    });
+                const int c = __popc(m);
+                int x = c;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, x, o);
+                    if (lane >= o) x += t;
                 }
+                __syncthreads();                 // earlier readers of wsum and sp are done
+                if (lane == 31) wsum[warp] = x;
+                __syncthreads();
+                int before = 0, all = 0;
+#pragma unroll
+                for (int v = 0; v < kTbThreads / 32; ++v) {
+                    if (v < warp) before += wsum[v];
+                    all += wsum[v];
+                }
+                if (ns + all > kTbCap) break;    // (never in the first round)
+                int pos = ns + before + x - c;
+                while (m) {
+                    sp[pos++] = (b << 20) | (k * 32 + __ffs(m) - 1);
+                    m &= m - 1;
+                }
+                ns += all;
+                w0 += kTbThreads;
             }
-            {
+            __syncthreads();
+            return w0;
+        };
+        int next = fill(0);
+        const bool whole = next >= nwords;       // one list holds the row's spikes
+        if (whole && ns == 0) continue;
+        // threads per synapse group: the row's synapses, rounded up to warps
+        int tc = 32;
+        while (tc < len && tc < kTbThreads) tc <<= 1;
+        const int slices = kTbThreads / tc, slice = tid / tc, tq = tid - slice * tc;
+        for (int qc = 0; qc < len; qc += tc) {
+            const int qi = qc + tq;
+            const uint32_t td = qi < len ? n.tgt_d[q0 + qi] : 0u;
+            const int j = (int)(td & 0xFFFFFFu), d = (int)(td >> 24);
+            const float *__restrict__ qj = n.qp + j;
+            float hi = 0.f, lo = 0.f;
+            if (!whole && qc > 0) next = fill(0);
+            for (;;) {
+                if (td != 0u) {
+#pragma unroll 4
+                    for (int c = slice; c < ns; c += slices) {
+                        const int v = sp[c];
+                        const int a = (v & 0xFFFFF) + d;
+                        const float x = a <= T ? __ldg(qj + ((long long)(v >> 20) * U + (a - 1)) * N) : 0.f;
+                        float e;
+                        two_sum(hi, x, hi, e);
+                        lo += e;
+                    }
+                }
+                if (next >= nwords) break;
+                next = fill(next);
+            }
+            if (slices > 1) {
+                red[tid] = make_float2(hi, lo);
+                __syncthreads();
+                if (slice == 0)
+                    for (int v = 1; v < slices; ++v) {
+                        const float2 o = red[v * tc + tq];
+                        float e;
+                        two_sum(hi, o.x, hi, e);
+                        lo += e + o.y;
+                    }
+                __syncthreads();
+            }
+            if (slice == 0 && td != 0u) {
+                const long long q = q0 + qi;
+                const float G = hi + lo;
                 const float w0 = n.w[q];
-                const float wn = window_update(n, q, w0, (float)G);
+                const float wn = window_update(n, q, w0, G);
                 if (!n.adam) n.w[q] = wn;
+                if (n.record_grad) n.grad[q] += n.inv_B * G;
             }
-            if (n.record_grad) n.grad[q] += n.inv_B * (float)G;
         }
-        __syncwarp();
     }
 }
 
@@ -1470,18 +1551,26 @@ void launch_filter_error(const Net &n, int i_end, cudaStream_t st) {
 }
 
 int launch_tables(const Net &n, int i_end, cudaStream_t st) {
-    const int bd = 128;
-    const dim3 grid((n.n_rec + bd - 1) / bd, n.B);
     const bool f64 = n.U > 128;          // long LIF windows sweep in FP64 (ALIF always does)
+    // blocks of one warp while blocks of four would leave SMs without work
+    // (four blocks per SM are resident)
+    const int bd = (long long)n.n_rec * n.B >= 128LL * 4 * 160 ? 128 : 32;
+    const dim3 grid((n.n_rec + bd - 1) / bd, n.B);
+#define EPROP_TAB(A, R, F)                                                                   \
+    do {                                                                                     \
+        if (n.has_state) tables_kernel<A, R, F, true><<<grid, bd, 0, st>>>(n, i_end);        \
+        else tables_kernel<A, R, F, false><<<grid, bd, 0, st>>>(n, i_end);                   \
+    } while (0)
     if (n.R_win) {
-        if (n.alif) tables_kernel<true, true, true><<<grid, bd, 0, st>>>(n, i_end);
-        else if (f64) tables_kernel<false, true, true><<<grid, bd, 0, st>>>(n, i_end);
-        else tables_kernel<false, true, false><<<grid, bd, 0, st>>>(n, i_end);
+        if (n.alif) EPROP_TAB(true, true, true);
+        else if (f64) EPROP_TAB(false, true, true);
+        else EPROP_TAB(false, true, false);
     } else {
-        if (n.alif) tables_kernel<true, false, true><<<grid, bd, 0, st>>>(n, i_end);
-        else if (f64) tables_kernel<false, false, true><<<grid, bd, 0, st>>>(n, i_end);
-        else tables_kernel<false, false, false><<<grid, bd, 0, st>>>(n, i_end);
+        if (n.alif) EPROP_TAB(true, false, true);
+        else if (f64) EPROP_TAB(false, false, true);
+        else EPROP_TAB(false, false, false);
     }
+#undef EPROP_TAB
     return 0;
 }
 
@@ -1543,10 +1632,8 @@ void launch_window_batched(const Net &n, int i_end, int sm_count, cudaStream_t s
 }
 
 void launch_trace_batched(const Net &n, int sm_count, cudaStream_t st) {
-    int blocks = (n.n_src + 7) / 8;
-    if (blocks > 8 * sm_count) blocks = 8 * sm_count;
-    if (n.alif) trace_batched_kernel<4><<<blocks, 256, 0, st>>>(n);
-    else trace_batched_kernel<2><<<blocks, 256, 0, st>>>(n);
+    const int blocks = n.n_src < 6 * sm_count ? n.n_src : 6 * sm_count;
+    trace_batched_kernel<<<blocks, kTbThreads, 0, st>>>(n);
 }
 
 void launch_readout_weights(const Net &n, int i_end, cudaStream_t st) {
