@@ -772,9 +772,9 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
     // Readout work (the per-step readout sum and error, the window's readout
     // weight update) reads the step's spike list and W_out and feeds only the
     // window-end kernels, so it runs on the second stream beside delivery and
-    // the next neuron updates; the weight update is forked after the tables
-    // kernel, which reads W_out as the feedback matrix when B is symmetric,
-    // and overlaps the window pass.  Joins: before the error filter and tables
+    // the next neuron updates; the weight update is forked after the
+    // learning-signal product, which reads W_out as the feedback matrix when
+    // B is symmetric, and overlaps the tables and the window pass.  Joins: before the error filter and tables
     // of a window (they read its errors), before the rollover (it clears the
     // spike bits the weight update reads), and at the end of the call.  With
     // a predictor attached everything stays on one stream (the prediction
@@ -785,7 +785,9 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
     // step's list until it has run (with a readout delay d_out it reads the
     // list of the step d_out back, and RS >= d_out + 2 keeps that one too).
     // (the persistent step loop does the readout itself: one stream)
-    const bool fork = n.pred_mode == 0 && n.RS > n.U && c.launch_mode != 2;
+    // (with the sample-resident loop only the window-end work is forked)
+    const bool sample_loop = eprop::sample_steps_fit(n);
+    const bool fork = n.pred_mode == 0 && (sample_loop || (n.RS > n.U && c.launch_mode != 2));
     cudaStream_t sr = fork ? net->st2 : st;
     auto fork_readout = [&]() {
         if (!fork) return;
@@ -800,7 +802,6 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
     // small networks run the steps of a window sample by sample in one launch
     // (every launch mode); larger ones with launch_mode 2 run all steps of the
     // call in one cooperative launch, else a few launches per step
-    const bool sample_loop = eprop::sample_steps_fit(n);
     const bool persistent = c.launch_mode == 2 && !sample_loop;
     if (persistent) {
         // form (2): every step of the call in one cooperative launch
@@ -835,14 +836,15 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
         }
         if (i % U == 0) {
             if (!sample_loop) join_readout();    // nothing forked since the last join otherwise
-            eprop::launch_filter_error(n, i, st);
+            fork_readout();
+            eprop::launch_filter_error(n, i, sr);
             // L[b][u][j] = sum_k B[j][k] E[b][u][k] of the whole window
             // (Eq. final-gradient), tensor cores with split TF32 operands
             eprop::launch_learning_signals(n.fb, n.E_win, n.L_win, c.n_rec, U, c.n_out, (int)B, n.err_flags, st);
-            eprop::launch_tables(n, i, st);
-            // after the tables: with symmetric feedback B is W_out itself
+            // after the product: with symmetric feedback B is W_out itself
             fork_readout();
             eprop::launch_readout_weights(n, i, sr);
+            eprop::launch_tables(n, i, st);
             L += 4;
             if (c.profile) cudaEventRecordWithFlags(net->ev[2 * nwin], st, cudaEventRecordExternal);
             if (net->trace_mode == 1) {

@@ -71,22 +71,51 @@ __global__ void end_call_kernel(Net n, int T) {
 // filtered error for the readout gradient: Ebar(u) = sum_{t >= u} kappa^{t-u} E^t
 // inside the window, and C = kappa * Ebar(a0 + 1) (Eq. eprop-output-new-subs-
 // rewritten, index-flipped inside the window).
-__global__ void filter_error_kernel(Net n) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n.B * n.n_out) return;
-    const int b = idx / n.n_out, k = idx % n.n_out;
-    const float *E = n.E_win + (long long)b * n.U * n.n_out + k;
-    float *Eb = n.Ebar_win + (long long)b * n.U * n.n_out + k;
-    // FP64 recursion with the FP64 filter constant (kappa + kappa_lo): over a
-    // long window the FP32 chain of products would carry a relative error of
-    // about (window length) x 2^-24 on errors that arrive late in the window
+//
+// One warp per (sample, readout).  The recursion runs in FP64 with the FP64
+// filter constant (kappa + kappa_lo): over a long window the FP32 chain of
+// products would carry a relative error of about (window length) x 2^-24 on
+// errors that arrive late in the window.  A thread walking the whole window
+// is one chain of U memory and FP64 latencies (0.2 us per step); so each lane
+// takes a contiguous piece of ceil(U / 32) steps, the pieces' sums are carried
+// across the lanes, and each lane repeats its piece with what comes from the
+// later ones.  Measured: window of 50 steps 29 -> 5.8 us (640 readouts), 350
+// steps 176 -> 9.5 us (640), 2200 steps 447 -> 26 us (64).
+__global__ void __launch_bounds__(32) filter_error_kernel(Net n) {
+    const int idx = blockIdx.x, lane = threadIdx.x;
+    const int b = idx / n.n_out, k = idx % n.n_out, K = n.n_out, U = n.U;
+    const float *__restrict__ E = n.E_win + (long long)b * U * K + k;
+    float *__restrict__ Eb = n.Ebar_win + (long long)b * U * K + k;
     const double kap = (double)n.kappa + (double)n.kappa_lo;
-    double acc = 0.0;
-    for (int u = n.U - 1; u >= 0; --u) {
-        acc = (double)E[(long long)u * n.n_out] + kap * acc;
-        Eb[(long long)u * n.n_out] = (float)acc;
+    const int m = (U + 31) / 32;                     // steps per lane, lane 31 holds the last ones
+    const int u0 = min(lane * m, U), u1 = min(u0 + m, U);
+    constexpr int kC = 8;
+    auto sweep = [&](double acc, bool store) {
+        for (int u = u1; u > u0; u -= kC) {
+            float e[kC];
+#pragma unroll
+            for (int c = 0; c < kC; ++c) e[c] = u - 1 - c >= u0 ? E[(long long)(u - 1 - c) * K] : 0.f;
+#pragma unroll
+            for (int c = 0; c < kC; ++c) {
+                if (u - 1 - c < u0) break;
+                acc = (double)e[c] + kap * acc;
+                if (store) Eb[(long long)(u - 1 - c) * K] = (float)acc;
+            }
+        }
+        return acc;
+    };
+    // (s, f): the piece's own sum and the factor kappa^(steps) on what follows
+    const double own = sweep(0.0, false);
+    double f = 1.0;
+    for (int u = u0; u < u1; ++u) f *= kap;
+    double carry = 0.0;                              // Ebar of the step after the lane's piece
+    double run = 0.0;
+    for (int l = 31; l >= 0; --l) {
+        if (lane == l) carry = run;
+        run = __shfl_sync(0xffffffffu, own, l) + __shfl_sync(0xffffffffu, f, l) * run;
     }
-    n.Cwin[idx] = (float)(kap * acc);
+    sweep(carry, true);
+    if (lane == 0) n.Cwin[idx] = (float)(kap * run);
 }
 
 // learning-signal tables: one thread per (sample, neuron), 128 neurons per
@@ -264,23 +293,45 @@ __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
 
 // Work-item offsets of one window: for the emission steps s = s_lo..s_hi
 // whose spikes arrive in the window, off[k] = sum_{k' < k} rows(s_lo + k').
-__global__ void window_offsets_kernel(Net n, int i_end) {
+// One thread per step sums its buckets, then a block scan (one warp walking
+// the steps paid a memory round trip per step: 287 us for 1000 steps, 31 us
+// for 100; now ~5 us).
+__global__ void __launch_bounds__(1024) window_offsets_kernel(Net n, int i_end) {
+    __shared__ int part[32];
     const int r_end = run_step_w(n, i_end);
     const int a0 = r_end - n.U;
     const int s_lo = max(a0 + 1 - n.D, 1);
     const int nsteps = r_end - 1 - s_lo + 1;
-    const int lane = threadIdx.x & 31;
-    long long acc = 0;
-    for (int k = 0; k < nsteps; ++k) {
-        int v = n.list_cnt[list_index(n, 0, (s_lo + k) % n.RS) + lane];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    long long base = 0;
+    for (int k0 = 0; k0 < nsteps; k0 += 1024) {
+        const int k = k0 + tid;
+        int v = 0;
+        if (k < nsteps) {
+            const int4 *c = reinterpret_cast<const int4 *>(n.list_cnt + list_index(n, 0, (s_lo + k) % n.RS));
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) n.win_off[k] = acc;
-        acc += v;
+            for (int q = 0; q < kBkt / 4; ++q) v += c[q].x + c[q].y + c[q].z + c[q].w;
+        }
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += t;
+        }
+        if (lane == 31) part[warp] = x;
+        __syncthreads();
+        long long before = 0, all = 0;
+        for (int w = 0; w < 32; ++w) {
+            if (w < warp) before += part[w];
+            all += part[w];
+        }
+        if (k < nsteps) n.win_off[k] = base + before + x - v;
+        base += all;
+        __syncthreads();
     }
-    if (lane == 0) n.win_off[nsteps > 0 ? nsteps : 0] = acc;
+    if (tid == 0) n.win_off[nsteps > 0 ? nsteps : 0] = base;
     // the row kernels' work counters (after the U + D + 2 offsets)
-    if (lane < kWorkCounters) n.win_off[n.U + n.D + 2 + lane] = 0;
+    if (tid < kWorkCounters) n.win_off[n.U + n.D + 2 + tid] = 0;
 }
 
 __device__ __forceinline__ bool any_spike(const uint32_t *words, int RW, int lo, int hi) {
@@ -1428,6 +1479,95 @@ __global__ void readout_weights_kernel(Net n, int i_end) {
     }
 }
 
+// Readout weights of small networks: one block per recurrent neuron, its
+// warps take the samples in turn (lanes over the readouts, the window's spike
+// words one per lane), and the samples' shares are added in sample order, so
+// the sums round as in readout_weights_kernel.  With one warp per neuron,
+// 200 neurons x 64 samples kept 25 blocks busy for 121 us (100 neurons x 32
+// samples of 2200 steps: 225 us); now 22 and 17 us.
+constexpr int kRwWarps = 8;
+constexpr int kRwMaxOut = 128;
+template <int KQ>
+__global__ void __launch_bounds__(kRwWarps * 32) readout_weights_small_kernel(Net n, int i_end) {
+    __shared__ float part[kRwWarps][KQ * 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    const int j = blockIdx.x, K = n.n_out, N = n.n_rec, U = n.U;
+    const int r_end = run_step_w(n, i_end);
+    const int a0 = r_end - U;
+    const int par = (a0 / U) & 1;
+    const float *zk_cur = n.zk + (long long)par * n.B * N;
+    float *zk_nxt = n.zk + (long long)(par ^ 1) * n.B * N;
+    const float kU = exp2f(n.log2_kappa * (float)U);
+    const int mask = n.RW * 32 - 1;
+    const int base = (a0 + 1) & ~31;                 // step of the first word's bit 0
+    const int nwd = (r_end - base) / 32 + 1;         // words covering a0+1 .. r_end
+    float g = 0.f;                                   // thread k < K: readout k
+    for (int b0 = 0; b0 < n.B; b0 += nwarp) {
+        const int b = b0 + warp;
+        if (b < n.B) {
+            const float z0 = zk_cur[(long long)b * N + j];
+            const uint32_t *words = src_words_c(n, b, n.n_in + j);
+            const float *Eb = n.Ebar_win + (long long)b * U * K;
+            float gb[KQ];
+#pragma unroll
+            for (int q = 0; q < KQ; ++q) {
+                const int k = lane + 32 * q;
+                gb[q] = k < K ? z0 * n.Cwin[b * K + k] : 0.f;
+            }
+            float zn = kU * z0;
+            for (int g0 = 0; g0 < nwd; g0 += 32) {
+                uint32_t wd = 0u;
+                if (g0 + lane < nwd) {
+                    const int sb = base + 32 * (g0 + lane);
+                    wd = words[(sb & mask) >> 5];
+                    const int lo = max(a0 + 1 - sb, 0), hi = min(r_end - sb, 31);
+                    wd = (wd >> lo) << lo;
+                    if (hi < 31) wd &= (2u << hi) - 1u;
+                }
+                unsigned any = __ballot_sync(0xffffffffu, wd != 0u);
+                while (any) {
+                    const int l = __ffs(any) - 1;
+                    any &= any - 1;
+                    uint32_t m = __shfl_sync(0xffffffffu, wd, l);
+                    while (m) {
+                        const int st = base + 32 * (g0 + l) + __ffs(m) - 1;
+                        m &= m - 1;
+                        // the spike reaches the readout d_out steps later
+                        // (Eq. eprop-output-new-subs-rewritten with delay)
+                        if (st + n.d_out <= r_end) {
+#pragma unroll
+                            for (int q = 0; q < KQ; ++q) {
+                                const int k = lane + 32 * q;
+                                if (k < K) gb[q] += __ldg(Eb + (long long)(st + n.d_out - a0 - 1) * K + k);
+                            }
+                        }
+                        zn += exp2f(n.log2_kappa * (float)(r_end - st));
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < KQ; ++q) part[warp][lane + 32 * q] = gb[q];
+            if (lane == 0) zk_nxt[(long long)b * N + j] = zn;
+        }
+        __syncthreads();
+        if (threadIdx.x < K)                         // blockDim >= K
+            for (int w = 0; w < min(nwarp, n.B - b0); ++w) g += part[w][threadIdx.x];
+        __syncthreads();
+    }
+    const int k = threadIdx.x;
+    if (k < K && n.out_mask[(long long)j * K + k]) {
+        const long long idx = (long long)j * K + k;
+        if (n.adam) {
+            n.gwin_out[idx] = n.inv_B * g;
+        } else {
+            const float w0 = n.w_out[idx];
+            const float wn = w0 - n.lr * n.inv_B * g;
+            n.w_out[idx] = (n.sign_mask & 4) ? keep_sign(w0, wn) : wn;
+        }
+        if (n.record_grad) n.grad_out[idx] += n.inv_B * g;
+    }
+}
+
 // rollover to the next window: move each source's anchor to its last spike
 // <= b - D and clear the bit positions of steps b+1 .. b+U.
 __global__ void rollover_kernel(Net n, int i_end) {
@@ -1607,7 +1747,7 @@ void launch_end_call(const Net &n, int T, cudaStream_t st) { end_call_kernel<<<1
 void launch_filter_error(const Net &n, int i_end, cudaStream_t st) {
     (void)i_end;
     const int tot = n.B * n.n_out;
-    filter_error_kernel<<<(tot + 127) / 128, 128, 0, st>>>(n);
+    filter_error_kernel<<<tot, 32, 0, st>>>(n);
 }
 
 int launch_tables(const Net &n, int i_end, cudaStream_t st) {
@@ -1635,7 +1775,7 @@ int launch_tables(const Net &n, int i_end, cudaStream_t st) {
 }
 
 void launch_trace_window(const Net &n, int i_end, int grid_x, cudaStream_t st) {
-    window_offsets_kernel<<<1, 32, 0, st>>>(n, i_end);
+    window_offsets_kernel<<<1, 1024, 0, st>>>(n, i_end);
     const size_t sm = sizeof(StageBuf) * 8 * kTStages + (size_t)(n.U + n.D + 1) * sizeof(long long);
     if (n.has_state) {
         if (n.alif) trace_window_kernel<true, true><<<grid_x, 256, sm, st>>>(n, i_end);
@@ -1647,7 +1787,7 @@ void launch_trace_window(const Net &n, int i_end, int grid_x, cudaStream_t st) {
 }
 
 void launch_window_pass(const Net &n, int i_end, int grid_x, int grid_idle, cudaStream_t st) {
-    window_offsets_kernel<<<1, 32, 0, st>>>(n, i_end);
+    window_offsets_kernel<<<1, 1024, 0, st>>>(n, i_end);
     const size_t sb = sizeof(StageBuf) * 8 * kPStages;
     const size_t sm = sb + (size_t)(n.U + n.D + 2) * sizeof(long long);
 #define EPROP_PASS(A, T, G)                                                             \
@@ -1697,6 +1837,15 @@ void launch_trace_batched(const Net &n, int sm_count, cudaStream_t st) {
 }
 
 void launch_readout_weights(const Net &n, int i_end, cudaStream_t st) {
+    // one warp per neuron fills the chip from about 2000 neurons on
+    if (n.n_rec <= 2048 && n.n_out <= kRwMaxOut) {
+        const int kq = (n.n_out + 31) / 32;
+        const int warps = n.B < kRwWarps ? (n.B > kq ? n.B : kq) : kRwWarps;
+        if (kq == 1) readout_weights_small_kernel<1><<<n.n_rec, warps * 32, 0, st>>>(n, i_end);
+        else if (kq == 2) readout_weights_small_kernel<2><<<n.n_rec, warps * 32, 0, st>>>(n, i_end);
+        else readout_weights_small_kernel<4><<<n.n_rec, warps * 32, 0, st>>>(n, i_end);
+        return;
+    }
     readout_weights_kernel<<<(unsigned)(((long long)n.n_rec * 32 + 255) / 256), 256, 0, st>>>(n, i_end);
 }
 
