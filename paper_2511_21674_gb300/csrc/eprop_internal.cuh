@@ -299,6 +299,47 @@ __device__ __forceinline__ void comp_step(float c_hi, float c_lo, float u_hi, fl
     x_hi = hi;
 }
 
+// Fixed point (2^-32) of a batch of weights and back, avoiding 64-bit
+// conversion instructions: float <-> 64-bit integer conversions take 16 cycles
+// per warp on an SM and 85 of latency (32-bit ones 2 and 34).  Both functions
+// give exactly the bits of those instructions: below 1 a weight's fixed point
+// is one 32-bit conversion, rounded to nearest even on the magnitude; a sum is
+// the error-free sum of its upper 40 and lower 24 bits, both exact in FP32, so
+// hi is the sum rounded to FP32 and lo the exact remainder.  Values outside
+// these ranges (and NaN) take the 64-bit instructions.  One range check per
+// batch keeps the batch's conversions independent of one another (a check per
+// weight serialised them and measured slower than the instruction).
+template <int M>
+__device__ __forceinline__ void to_fixed(const float (&w)[M], long long (&fx)[M]) {
+    bool small = true;
+#pragma unroll
+    for (int u = 0; u < M; ++u) small &= fabsf(w[u]) < 1.0f;
+    if (small) {
+#pragma unroll
+        for (int u = 0; u < M; ++u) {
+            const long long m = (long long)__float2uint_rn(fabsf(w[u]) * 4294967296.0f);
+            fx[u] = w[u] < 0.0f ? -m : m;
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < M; ++u) fx[u] = __float2ll_rn(w[u] * 4294967296.0f);
+    }
+}
+__device__ __forceinline__ void fixed_to_pair(long long acc, float &hi, float &lo) {
+    const long long up = acc >> 24;
+    if (up >= -(1LL << 24) && up < (1LL << 24)) {
+        const float f1 = (float)(int)up * 16777216.0f;
+        const float f0 = (float)(int)((unsigned)acc & 0xFFFFFFu);
+        const float s = __fadd_rn(f1, f0);
+        hi = s * kFixInv;
+        lo = __fsub_rn(f0, __fsub_rn(s, f1)) * kFixInv;
+    } else {
+        const float s = (float)acc;
+        hi = s * kFixInv;
+        lo = (float)(acc - (long long)s) * kFixInv;
+    }
+}
+
 __device__ __forceinline__ uint64_t mix64(uint64_t x) {
     // SplitMix64 output function (Steele, Lea & Flood 2014)
     uint64_t z = x + 0x9E3779B97F4A7C15ULL;

@@ -724,13 +724,14 @@ __global__ void __launch_bounds__(256, 4) deliver_band_kernel(Net n, int i) {
                 tdv[u] = in ? n.bd_td[q] : kBandPad;
                 wv[u] = in ? n.w[q] : 0.f;
             }
+            long long fx[4];
+            to_fixed(wv, fx);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (tdv[u] == kBandPad) continue;
                 const int j = bm[u] * n.band_w + (int)(tdv[u] & 0x3FFFu);
                 const int dl = (int)((tdv[u] >> 14) & 7u) + 1;
-                const long long fx = __float2ll_rn(wv[u] * 4294967296.0f);
-                atomicAdd(reinterpret_cast<unsigned long long *>(&n.ring[ring_off[dl] + j]), (unsigned long long)fx);
+                atomicAdd(reinterpret_cast<unsigned long long *>(&n.ring[ring_off[dl] + j]), (unsigned long long)fx[u]);
             }
         }
     }

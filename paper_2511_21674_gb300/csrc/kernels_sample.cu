@@ -64,7 +64,7 @@ __host__ __device__ inline SampleShape sample_shape(int n_in, int n_rec, int n_o
 }
 
 static size_t sample_smem(const SampleShape &s) {
-    size_t b = (size_t)s.R * s.NP * 8;                        // ring words
+    size_t b = ((size_t)s.R * s.NP + 32) * 8;                 // ring words and a spare one per lane
     b += (size_t)3 * s.NP * sizeof(int4);                     // spike lists of three steps
     if (s.KI) {
         b += (size_t)2 * kSmpInCap * (sizeof(int4) + sizeof(int));   // input rows and ids of two steps
@@ -77,13 +77,34 @@ __device__ __forceinline__ void bar_sync(int id, int threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
-// adds the fixed-point value of weight w to a ring entry
-__device__ __forceinline__ void ring_add(uint32_t *lo, uint32_t *hi, float w) {
-    const long long fx = __float2ll_rn(w * 4294967296.0f);
-    const uint32_t l = (uint32_t)fx;
-    const uint32_t old = atomicAdd(lo, l);
-    const uint32_t h = (uint32_t)((unsigned long long)fx >> 32) + (old + l < l ? 1u : 0u);
-    if (h) atomicAdd(hi, h);
+// Adds up to 32 M records of a row to the ring (one warp).  No branch per
+// record: absent ones add zero to the warp's spare words, so the conversions
+// and the atomics of the batch overlap.
+template <int M>
+__device__ __forceinline__ void add_records(const Net &n, int start, int cnt, int i, int smask, int NP, int spare,
+                                            uint32_t *ring_lo, uint32_t *ring_hi) {
+    const int lane = threadIdx.x & 31;
+    uint32_t td[M];
+    float wv[M];
+#pragma unroll
+    for (int u = 0; u < M; ++u) {
+        const int k = lane + 32 * u;
+        td[u] = k < cnt ? __ldg(n.tgt_d + start + k) : 0u;
+        wv[u] = k < cnt ? __ldg(n.w + start + k) : 0.f;
+    }
+    long long fx[M];
+    to_fixed(wv, fx);
+    int o[M];
+    uint32_t old[M];
+#pragma unroll
+    for (int u = 0; u < M; ++u)
+        o[u] = td[u] ? ((i + (int)(td[u] >> 24)) & smask) * NP + (int)(td[u] & 0xFFFFFFu) : spare;
+#pragma unroll
+    for (int u = 0; u < M; ++u) old[u] = atomicAdd(ring_lo + o[u], (uint32_t)fx[u]);
+#pragma unroll
+    for (int u = 0; u < M; ++u)
+        atomicAdd(ring_hi + o[u],
+                  (uint32_t)((unsigned long long)fx[u] >> 32) + (old[u] + (uint32_t)fx[u] < old[u] ? 1u : 0u));
 }
 
 template <bool VAR, int NPT, int BT>
@@ -97,8 +118,8 @@ __global__ void __launch_bounds__(BT, 1) sample_steps_kernel(Net n, int i0, int 
     __shared__ float red_s[4];
     const SampleShape sh = sample_shape(n.n_in, n.n_rec, n.n_out, n.D);
     uint32_t *ring_lo = reinterpret_cast<uint32_t *>(dsm);
-    uint32_t *ring_hi = ring_lo + sh.R * sh.NP;
-    int4 *slist = reinterpret_cast<int4 *>(ring_hi + sh.R * sh.NP);
+    uint32_t *ring_hi = ring_lo + sh.R * sh.NP + 32;
+    int4 *slist = reinterpret_cast<int4 *>(ring_hi + sh.R * sh.NP + 32);
     int4 *xrow = slist + 3 * sh.NP;
     int *xid = reinterpret_cast<int *>(xrow + 2 * kSmpInCap);
     uint32_t *xbit = reinterpret_cast<uint32_t *>(xid + 2 * kSmpInCap);
@@ -110,7 +131,7 @@ __global__ void __launch_bounds__(BT, 1) sample_steps_kernel(Net n, int i0, int 
     const int i_last = min(i1, len);
     const int rmask = n.RW * 32 - 1;
     const long long nb0 = (long long)b * N;
-    const int D1 = D + 1, smask = sh.R - 1;
+    const int D1 = D + 1, smask = sh.R - 1, spare = sh.R * sh.NP + lane;
     long long *ring_g = n.ring + (long long)b * D1 * N;
 
     if (i0 <= i_last) {
@@ -118,7 +139,7 @@ __global__ void __launch_bounds__(BT, 1) sample_steps_kernel(Net n, int i0, int 
         for (int m = tid; m < n.n_thr; m += BT) thr_s[m] = n.drive_thr[m];
         if (tid < 3) cnt_s[tid] = 0;
         if (tid < 4 * kBkt) bcnt_s[tid >> 5][tid & 31] = 0;
-        for (int q = tid; q < 2 * sh.R * sh.NP; q += BT) ring_lo[q] = 0;
+        for (int q = tid; q < 2 * (sh.R * sh.NP + 32); q += BT) ring_lo[q] = 0;
         if (sh.KI)
             for (int q = tid; q < 2 * sh.in_words; q += BT) xbit[q] = 0;
         __syncthreads();
@@ -134,22 +155,12 @@ __global__ void __launch_bounds__(BT, 1) sample_steps_kernel(Net n, int i0, int 
         __syncthreads();
         unsigned long long ev = 0;
 
-        // rows of delivery items, one warp per item: records [q, q + cnt), cnt <= kSmpPart
+        // one delivery item (one warp): records [start, start + cnt), cnt <= kSmpPart
         auto deliver = [&](int start, int cnt, int i) {
-            uint32_t td[kSmpPart / 32];
-            float wv[kSmpPart / 32];
-#pragma unroll
-            for (int u = 0; u < kSmpPart / 32; ++u) {
-                const int k = lane + 32 * u;
-                td[u] = k < cnt ? __ldg(n.tgt_d + start + k) : 0u;
-                wv[u] = k < cnt ? __ldg(n.w + start + k) : 0.f;
-            }
-#pragma unroll
-            for (int u = 0; u < kSmpPart / 32; ++u) {
-                if (td[u] == 0u) continue;       // no record (delays are >= 1)
-                const int o = ((i + (int)(td[u] >> 24)) & smask) * sh.NP + (int)(td[u] & 0xFFFFFFu);
-                ring_add(ring_lo + o, ring_hi + o, wv[u]);
-            }
+            if (cnt <= kSmpPart / 2)
+                add_records<kSmpPart / 64>(n, start, cnt, i, smask, sh.NP, spare, ring_lo, ring_hi);
+            else
+                add_records<kSmpPart / 32>(n, start, cnt, i, smask, sh.NP, spare, ring_lo, ring_hi);
         };
 
         if (warp < NW) {
@@ -338,8 +349,12 @@ __global__ void __launch_bounds__(BT, 1) sample_steps_kernel(Net n, int i0, int 
             const long long bk = (long long)b * K + (has_k ? k : 0);
             float y = has_k ? n.y[bk] : 0.f;
             float loss = k == 0 ? n.loss_acc[b] : 0.f;
+            // lanes at and past K hold the neutral element: with few readouts
+            // the wider exchanges change nothing (the first lanes have the result)
+            int width = 16;
+            while (sh.KR == 1 && width >= K && width > 1) width >>= 1;
             auto reduce = [&](float x, bool mx) -> float {
-                for (int o = 16; o > 0; o >>= 1) {
+                for (int o = width; o > 0; o >>= 1) {
                     const float v = __shfl_xor_sync(0xffffffffu, x, o);
                     x = mx ? fmaxf(x, v) : x + v;
                 }
@@ -354,26 +369,36 @@ __global__ void __launch_bounds__(BT, 1) sample_steps_kernel(Net n, int i0, int 
             auto load_tgt = [&](int i) {
                 return (has_k && i <= i_last) ? n.targets[((long long)b * T + (i - 1)) * K + k] : 0.f;
             };
-            auto load_win = [&](int i) {
-                return (n.window && i <= i_last) ? (float)n.window[(long long)b * T + (i - 1)] : 1.0f;
+            auto load_win = [&](int i) -> int {  // (converted where it is used, a step later)
+                return i <= i_last ? n.window[(long long)b * T + (i - 1)] : 0;
             };
-            float tgt = load_tgt(i0), win = load_win(i0);
+            float tgt = load_tgt(i0);
+            int win = load_win(i0);
             auto finish = [&](int i) {           // readout of step i (its spike list is complete)
-                const float tgt_n = load_tgt(i + 1), win_n = load_win(i + 1);
+                const float tgt_n = load_tgt(i + 1);
+                const int win_n = load_win(i + 1);
                 const int c = cnt_s[i % 3];
                 const int4 *lst = slist + (i % 3) * sh.NP;
                 long long acc = 0;
                 if (has_k) {
-#pragma unroll 4
-                    for (int e = 0; e < c; ++e)
-                        acc += __float2ll_rn(__ldg(n.w_out + (long long)lst[e].x * K + k) * 4294967296.0f);
+                    constexpr int kC = 4;
+                    for (int e = 0; e < c; e += kC) {
+                        float wv[kC];
+                        long long fx[kC];
+#pragma unroll
+                        for (int u = 0; u < kC; ++u)
+                            wv[u] = e + u < c ? __ldg(n.w_out + (long long)lst[e + u].x * K + k) : 0.f;
+                        to_fixed(wv, fx);
+#pragma unroll
+                        for (int u = 0; u < kC; ++u) acc += fx[u];
+                    }
                 }
                 if (has_k) {
                     y = readout_step(n, y, acc);
                     n.y_rec[((long long)b * T + (i - 1)) * K + k] = y;
                 }
                 float E;
-                const float l = error_signal(n, y, tgt, win, has_k, E, [&](float x) { return reduce(x, true); },
+                const float l = error_signal(n, y, tgt, (float)win, has_k, E, [&](float x) { return reduce(x, true); },
                                              [&](float x) { return reduce(x, false); });
                 if (has_k) n.E_win[((long long)b * U + (i - i0)) * K + k] = E;
                 const float tot = reduce(l, false);

@@ -514,14 +514,15 @@ __global__ void __launch_bounds__(256, STATE ? 2 : 4) deliver_kernel(Net n, int 
                     wv[u] -= n.lr * G;
                 }
             }
+            long long fx[4];
+            to_fixed(wv, fx);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (td[u] == 0u) continue;
                 const int j = (int)(td[u] & 0xFFFFFFu);
                 const int dl = (int)(td[u] >> 24);
-                const long long fx = __float2ll_rn(wv[u] * 4294967296.0f);
                 atomicAdd(reinterpret_cast<unsigned long long *>(&ring_b[ring_off[dl] + j]),
-                          (unsigned long long)fx);
+                          (unsigned long long)fx[u]);
             }
         }
         __syncwarp();

@@ -25,9 +25,8 @@ template <bool VAR>
 __device__ __forceinline__ void neuron_core(const Net &n, int b, int j, long long t_abs, const uint32_t *thr_s,
                                             long long acc_q, int forced_z, NeuronRegs &s, float &psi, int &z) {
     // exact fixed-point input split into an FP32 pair
-    const float acc_hi = (float)acc_q;
-    float u_hi = acc_hi * kFixInv;
-    float u_lo = (float)(acc_q - (long long)acc_hi) * kFixInv;
+    float u_hi, u_lo;
+    fixed_to_pair(acc_q, u_hi, u_lo);
     if (n.n_thr > 0) {
         const uint64_t h = mix64(mix64(mix64(n.drive_seed ^ (uint64_t)j) ^ (uint64_t)t_abs) ^ (uint64_t)b);
         const uint32_t u = (uint32_t)(h >> 32);
@@ -96,7 +95,9 @@ __device__ __forceinline__ float rate_signal(const Net &n, float rate) {
 // Leaky readout (Eq. leaky_integrator): y' = kappa y + input, the input
 // summed in fixed point
 __device__ __forceinline__ float readout_step(const Net &n, float y, long long acc) {
-    return __fmaf_rn((float)acc, kFixInv, __fmul_rn(n.kappa, y));
+    float in, rest;                      // in = the sum rounded to FP32
+    fixed_to_pair(acc, in, rest);
+    return __fadd_rn(in, __fmul_rn(n.kappa, y));
 }
 
 // Error signal E_k and this readout's share of the step's loss (Eq. mean-
