@@ -118,21 +118,64 @@ __global__ void __launch_bounds__(32) filter_error_kernel(Net n) {
     if (lane == 0) n.Cwin[idx] = (float)(kap * run);
 }
 
-// learning-signal tables: one thread per (sample, neuron), 128 neurons per
-// block.  The window is swept backwards in chunks of steps: the chunk's
-// learning signals L^t = sum_k B_jk E_k^t (Eq. final-gradient; formed for
-// the whole window beforehand on the tensor cores, L_win) are
-// loaded into registers, then the adjoint recursion writes the per-step
-// tables and, at the window start, the window coefficients.
+// FP32 pairs h + l (|l| about half an ulp of h): about 48 bits.  The products
+// and sums are built from error-free FP32 operations (TwoProduct through the
+// FMA, Knuth's TwoSum; Dekker 1971), spelled out with explicit rounding.
+struct Pair {
+    float h, l;
+};
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
+    const float p = __fmul_rn(a.h, b.h);
+    return {p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ Pair pair_mul(Pair a, float b) {
+    const float p = __fmul_rn(a.h, b);
+    return {p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p))};
+}
+__device__ __forceinline__ Pair pair_norm(float s, float e) {        // |e| small against s
+    const float h = __fadd_rn(s, e);
+    return {h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
+    const float s = __fadd_rn(a.h, b.h), bb = __fsub_rn(s, a.h);
+    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fsub_rn(b.h, bb));
+    return pair_norm(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ Pair pair_add(Pair a, float b) { return pair_add(a, Pair{b, 0.f}); }
+__device__ __forceinline__ Pair pair_neg(Pair a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ float pair_float(Pair a) { return __fadd_rn(a.h, a.l); }
+
+// the same operations on one float, so one sweep serves both
+__device__ __forceinline__ float pair_mul(float a, float b) { return a * b; }
+__device__ __forceinline__ float pair_add(float a, float b) { return a + b; }
+__device__ __forceinline__ float pair_float(float a) { return a; }
+
+// learning-signal tables: one thread per (sample, neuron).  The window is
+// swept backwards in chunks of steps: the chunk's learning signals L^t =
+// sum_k B_jk E_k^t (Eq. final-gradient; formed for the whole window beforehand
+// on the tensor cores, L_win) are loaded into registers, then the adjoint
+// recursion writes the per-step tables and, at the window start, the window
+// coefficients.
 // STATE: the window's end state and coefficients are wanted (carried traces).
 // Without carried state nothing reads them: only Q is swept and written, one
 // float per step and neuron.
-// The FP64 sweep is bound by an SM's FP64 pipe (2 lanes per clock: a warp
-// instruction takes 16 cycles), so the host deals it in blocks of one warp
-// until every SM has several: 100 neurons x 1000 steps 1226 us
-// in one block of four warps, 736 us in four blocks.
-template <bool ALIF, bool REG, bool F64, bool STATE>
+// PAIR: the sweep is the per-window reduction of the gradient.  For ALIF the
+// eligibility psi (zbar - beta eps_a) is a near-cancellation of two
+// long-memory traces (FP32 loses up to 1e-1 relative on some elements over a
+// few hundred steps), and over more than 128 steps the FP32 chain of decays
+// carries a relative error of about (steps) x 2^-24; those sweeps run in FP32
+// pairs, short LIF windows in FP32.  FP64 served them before: an SM has 2
+// FP64 lanes, so a warp instruction takes 64 cycles of its sub-partition and
+// the sweep was bound by that pipe.  With the pairs' ~90 FP32 operations per
+// step it is bound by their dependence chain; blocks of one warp spread small
+// networks over all SMs.  Measured (FP64 in blocks of one warp -> pairs; the
+// FP64 form in blocks of 128 in brackets): 100 LIF x 1000 steps [1226] 736 ->
+// 126 us, 64 samples x 200 ALIF x 350 steps 313 -> 57 us, 32 x 100 x 2200 steps
+// 1915 -> 337 us, 64 x 200 x 50 steps with carried state 83 -> 23 us.  Against
+// 64-bit gradients the errors are those of the FP64 sweep (4e-7 and below).
+template <bool ALIF, bool REG, bool PAIR, bool STATE>
 __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
+    static_assert(PAIR || !ALIF, "the ALIF sweep needs pairs");
     constexpr int kTC = ALIF ? 16 : 32;     // window steps per chunk
     const int b = blockIdx.y;
     const int U = n.U, N = n.n_rec;
@@ -147,28 +190,44 @@ __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
     // signal R^t (Eq. ema-gradient); its adjoint mb joins me wherever the
     // eligibility e^t enters (e^t feeds both filters)
     const float *R_g = REG ? n.R_win + (long long)b * U * N + (act ? j : 0) : nullptr;
-    // The adjoint sweep is the per-window reduction of the gradient.  For
-    // ALIF the eligibility psi (zbar - beta eps_a) is a near-cancellation of
-    // two long-memory traces, so the sweep runs in FP64 there (FP32 loses up
-    // to 1e-1 relative on some elements over a few hundred steps); the LIF
-    // sweep has no such cancellation and runs in FP32.
-    // Long LIF windows (more than 128 steps) sweep in FP64 as well: the FP32
-    // chain of decays carries a relative error of about (steps) x 2^-24 on
-    // the contributions of early arrivals.
-    using R = typename std::conditional<ALIF || F64, double, float>::type;
-    const R alpha = (R)n.alpha + (R)n.alpha_lo;
-    const R rho = ALIF ? (R)n.rho + (R)n.rho_lo : (R)0;
-    const R beta = n.beta_a;
-    // kappa_e^m over a window of hundreds of steps: in the FP64 sweep the
-    // filter constant keeps its FP64 value (hi + lo), as alpha and rho do
-    const R ke = (ALIF || F64) ? (R)n.kappa_e + (R)n.kappa_e_lo : (R)n.kappa_e;
+    using R = typename std::conditional<PAIR, Pair, float>::type;
+    auto constant = [](float hi, float lo) -> R {
+        if constexpr (PAIR) return Pair{hi, lo};
+        else return hi;
+    };
+    const R zero = constant(0.f, 0.f), one = constant(1.f, 0.f);
+    const R alpha = constant(PAIR ? n.alpha : n.alpha + n.alpha_lo, n.alpha_lo);
+    const R rho = constant(n.rho, n.rho_lo);
+    const R ke = constant(n.kappa_e, n.kappa_e_lo);
+    const float beta = n.beta_a;
     // adjoint of G (mz, ma, me); of ebar^b (ez, ea, ee); of eps_a^b (az, aa, ae)
-    R mz = 0, ma = 0, me = 0;
-    R ez = 0, ea = 0, ee = 1;
-    R az = 0, aa = 1, ae = 0;
-    R pn = 0;
-    R mb = 0;                                  // adjoint of F_beta(e) (regularisation)
-    const R breg = (R)n.beta_reg;
+    R mz = zero, ma = zero, me = zero;
+    R ez = zero, ea = zero, ee = one;
+    R az = zero, aa = one, ae = zero;
+    R mb = zero;                               // adjoint of F_beta(e) (regularisation)
+    float pn = 0.f;
+    // x -> (A^{u+1})^T x with A^{u+1} from psi^u = p, psi^{u+1} = pn; D =
+    // adjoint of e^{u+1} (both filters of the eligibility).  With X = pn D and
+    // Y = xa - beta X:  xz' = alpha (xz + X) + p Y,  xa' = (rho - beta p) Y.
+    auto back = [&](R &xz, R &xa, R D, float p, float pn1, R g2) {
+        if constexpr (PAIR) {
+            const R X = pair_mul(D, pn1);
+            const R W = pair_mul(pair_add(xz, X), alpha);
+            if (ALIF) {
+                const R Y = pair_add(xa, pair_neg(pair_mul(X, beta)));
+                xz = pair_add(W, pair_mul(Y, p));
+                xa = pair_mul(Y, g2);
+            } else {
+                xz = W;
+            }
+        } else {
+            xz = alpha * xz + alpha * pn1 * D;   // short LIF windows
+        }
+    };
+    auto adapt = [&](float p) -> R {           // rho - beta p
+        if constexpr (PAIR) return pair_add(rho, pair_neg(pair_mul(Pair{p, 0.f}, beta)));
+        else return rho;
+    };
     const float psi_b = act ? psi_g[(long long)U * N] : 0.f;
     // generalized delays (one window per call): step u pairs with the
     // learning signal of u + d_out, which reaches the neuron only if it was
@@ -201,48 +260,34 @@ __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
         for (int c = 0; c < kTC; ++c) {
             const int u = u1 - c;
             if (u < u0) break;
-            const R p = Pc[c];                               // psi^{a0+u}
+            const float p = Pc[c];                           // psi^{a0+u}
             if (u < U) {
-                // x -> (A^{u+1})^T x with A^{u+1} from psi^u = p, psi^{u+1} = pn;
-                // D = adjoint of e^{u+1} (both filters of the eligibility)
-                const R D = REG ? me + mb : me;
-                if (REG) mb = breg * mb;
-                if (ALIF) {
-                    const R g1 = alpha - beta * p, g2 = rho - beta * p;
-                    R nz = alpha * mz + p * ma + pn * g1 * D;
-                    R na = g2 * ma - beta * pn * g2 * D;
-                    R ne = ke * me;
-                    mz = nz; ma = na; me = ne;
-                    if (STATE) {
-                        nz = alpha * ez + p * ea + pn * g1 * ee;
-                        na = g2 * ea - beta * pn * g2 * ee;
-                        ne = ke * ee;
-                        ez = nz; ea = na; ee = ne;
-                        nz = alpha * az + p * aa + pn * g1 * ae;
-                        na = g2 * aa - beta * pn * g2 * ae;
-                        ne = ke * ae;
-                        az = nz; aa = na; ae = ne;
-                    }
-                } else {
-                    mz = alpha * mz + alpha * pn * D;
-                    me = ke * me;
-                    if (STATE) {
-                        ez = alpha * ez + alpha * pn * ee;
-                        ee = ke * ee;
+                const R g2 = ALIF ? adapt(p) : zero;
+                back(mz, ma, REG ? pair_add(me, mb) : me, p, pn, g2);
+                me = pair_mul(me, ke);
+                if (REG) mb = pair_mul(mb, n.beta_reg);
+                if (STATE) {
+                    back(ez, ea, ee, p, pn, g2);
+                    ee = pair_mul(ee, ke);
+                    if (ALIF) {
+                        back(az, aa, ae, p, pn, g2);
+                        ae = pair_mul(ae, ke);
                     }
                 }
             }
-            me += (R)Lc[c];
-            if (REG) mb += (R)Rc[c];
-            const R De = REG ? me + mb : me;           // adjoint of e^u
+            me = pair_add(me, Lc[c]);
+            if (REG) mb = pair_add(mb, Rc[c]);
+            const R De = REG ? pair_add(me, mb) : me;        // adjoint of e^u
+            const float Q = pair_float(pair_add(mz, pair_mul(De, p)));
             if (!STATE) {
-                n.qp[qbase + (long long)(u - 1) * N] = (float)(mz + p * De);
+                n.qp[qbase + (long long)(u - 1) * N] = Q;
             } else if (ALIF) {
                 reinterpret_cast<float4 *>(n.qp)[qbase + (long long)(u - 1) * N] =
-                    make_float4((float)(mz + p * De), (float)(ez + p * ee), (float)(az + p * ae), 0.f);
+                    make_float4(Q, pair_float(pair_add(ez, pair_mul(ee, p))), pair_float(pair_add(az, pair_mul(ae, p))),
+                                0.f);
             } else {
                 reinterpret_cast<float2 *>(n.qp)[qbase + (long long)(u - 1) * N] =
-                    make_float2((float)(mz + p * De), (float)(ez + p * ee));
+                    make_float2(Q, pair_float(pair_add(ez, pair_mul(ee, p))));
             }
             pn = p;
         }
@@ -250,28 +295,12 @@ __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
             // step a0 (u = 0): the window coefficients c = (A^{a0+1})^T mu^{a0+1}
             // (regularisation runs without carried state: no coefficients
             // of F_beta are kept, only G's adjoint sees it)
-            const R p = Pc[kTC];
-            const R D = REG ? me + mb : me;
-            if (ALIF) {
-                const R g1 = alpha - beta * p, g2 = rho - beta * p;
-                R nz = alpha * mz + p * ma + pn * g1 * D;
-                R na = g2 * ma - beta * pn * g2 * D;
-                R ne = ke * me;
-                mz = nz; ma = na; me = ne;
-                nz = alpha * ez + p * ea + pn * g1 * ee;
-                na = g2 * ea - beta * pn * g2 * ee;
-                ne = ke * ee;
-                ez = nz; ea = na; ee = ne;
-                nz = alpha * az + p * aa + pn * g1 * ae;
-                na = g2 * aa - beta * pn * g2 * ae;
-                ne = ke * ae;
-                az = nz; aa = na; ae = ne;
-            } else {
-                mz = alpha * mz + alpha * pn * D;
-                me = ke * me;
-                ez = alpha * ez + alpha * pn * ee;
-                ee = ke * ee;
-            }
+            const float p = Pc[kTC];
+            const R g2 = ALIF ? adapt(p) : zero;
+            back(mz, ma, me, p, pn, g2);
+            me = pair_mul(me, ke);
+            back(ez, ea, ee, p, pn, g2);
+            if (ALIF) back(az, aa, ae, p, pn, g2);
         }
     }
     if (!act) return;
@@ -282,10 +311,10 @@ __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
         const long long cj = ((long long)b * N + j) * n.RC + slot;
         if (ALIF) {
             float4 *c = reinterpret_cast<float4 *>(n.coef) + cj * 2;
-            c[0] = make_float4((float)mz, (float)ma, (float)me, (float)az);
-            c[1] = make_float4((float)aa, (float)ez, (float)ea, 0.f);
+            c[0] = make_float4(pair_float(mz), pair_float(ma), pair_float(me), pair_float(az));
+            c[1] = make_float4(pair_float(aa), pair_float(ez), pair_float(ea), 0.f);
         } else {
-            reinterpret_cast<float4 *>(n.coef)[cj] = make_float4((float)mz, (float)me, (float)ez, 0.f);
+            reinterpret_cast<float4 *>(n.coef)[cj] = make_float4(pair_float(mz), pair_float(me), pair_float(ez), 0.f);
         }
     }
     n.psi_hist[(long long)b * (U + 1) * N + j] = psi_b;     // slot 0 of the next window
@@ -1751,7 +1780,7 @@ void launch_filter_error(const Net &n, int i_end, cudaStream_t st) {
 }
 
 int launch_tables(const Net &n, int i_end, cudaStream_t st) {
-    const bool f64 = n.U > 128;          // long LIF windows sweep in FP64 (ALIF always does)
+    const bool pair = n.U > 128;         // long LIF windows sweep in FP32 pairs (ALIF always does)
     // blocks of one warp while blocks of four would leave SMs without work
     // (four blocks per SM are resident)
     const int bd = (long long)n.n_rec * n.B >= 128LL * 4 * 160 ? 128 : 32;
@@ -1763,11 +1792,11 @@ int launch_tables(const Net &n, int i_end, cudaStream_t st) {
     } while (0)
     if (n.R_win) {
         if (n.alif) EPROP_TAB(true, true, true);
-        else if (f64) EPROP_TAB(false, true, true);
+        else if (pair) EPROP_TAB(false, true, true);
         else EPROP_TAB(false, true, false);
     } else {
         if (n.alif) EPROP_TAB(true, false, true);
-        else if (f64) EPROP_TAB(false, false, true);
+        else if (pair) EPROP_TAB(false, false, true);
         else EPROP_TAB(false, false, false);
     }
 #undef EPROP_TAB
