@@ -827,7 +827,7 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
             if (n.pred_mode & 1) {
                 n.pred_y = predictor_issue_forward(net->pred, n.pred_x, (int)B, st);
                 eprop::launch_pred_apply(n, i, st);
-                L += 5;
+                L += 2;
             }
         }
         if (n.band) eprop::launch_deliver_band(n, i, deliver_rows, st);

@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -22,9 +23,15 @@ struct eprop_predictor {
     cudaStream_t st = nullptr;
     int own_stream = 0;
     float *params = nullptr, *grads = nullptr, *m = nullptr, *v = nullptr;
+    // BF16 arrays have rows padded to multiples of 8 values (16-byte pieces)
+    int ldX = 0, ldH = 0, ldK = 0;
     bf16 *Wh[3] = {nullptr, nullptr, nullptr};
     bf16 *Xh = nullptr, *H1h = nullptr, *H2h = nullptr, *dYh = nullptr, *dA2h = nullptr, *dA1h = nullptr;
-    float *A1 = nullptr, *A2 = nullptr, *Y = nullptr, *dYf = nullptr, *dA2f = nullptr, *dA1f = nullptr;
+    float *A1 = nullptr, *A2 = nullptr, *Y = nullptr;
+    float *gpart = nullptr;          // [kMaxSlices][n_params] weight gradients of row slices
+    float *bpart = nullptr;          // [row tiles][2 hidden + n_out] bias gradients of row tiles
+    float *lpart = nullptr;          // [row tiles] squared errors
+    int sm_count = 1, max_slices = 1;
     float *xin = nullptr, *ein = nullptr, *yout = nullptr, *loss = nullptr;
     float *stage = nullptr;          // FP32 widening of BF16 buffers for eprop_predictor_read
     float *in_scale = nullptr;       // [n_in] input scale (part of the model; default 1)
@@ -43,164 +50,397 @@ __device__ __forceinline__ float gelu_grad(float x) {
     return 0.5f * erfcf(-x * 0.70710678118654752f) + x * expf(-0.5f * x * x) * 0.39894228040143268f;
 }
 
-// inputs: x * scale[column], rounded to BF16
-__global__ void input_bf16_kernel(const float *src, const float *scale, int cols, bf16 *dst, long long n) {
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
-         q += (long long)gridDim.x * blockDim.x)
-        dst[q] = __float2bfloat16_rn(src[q] * scale[q % cols]);
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// 16-byte asynchronous copy; zeros when !in
+__device__ __forceinline__ void cp16(void *dst, const void *src, bool in) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(in ? 16 : 0)
+                 : "memory");
 }
-
-__global__ void to_bf16_kernel(const float *src, bf16 *dst, long long n) {
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
-         q += (long long)gridDim.x * blockDim.x)
-        dst[q] = __float2bfloat16_rn(src[q]);
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void ldm4(uint32_t (&r)[4], const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(p)) : "memory");
 }
-
-// A(m, k) = A[m * sam + k * sak], B(k, n) = B[k * sbk + n * sbn]
-struct Gemm {
-    const bf16 *A, *B;
-    long long sam, sak, sbk, sbn;
-    int M, N, K;
-    const float *bias;      // [N] or null
-    const float *pre;       // [M][N] pre-activation for the GELU derivative
-    float *outF;            // [M][N]
-    bf16 *outH;             // [M][N]
-};
-
-enum { EPI_STORE = 0, EPI_BIAS = 1, EPI_BIAS_GELU = 2, EPI_DGELU = 3 };
-
-__device__ __forceinline__ uint32_t pack2(bf16 lo, bf16 hi) {
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+__device__ __forceinline__ void ldm4t(uint32_t (&r)[4], const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(p)) : "memory");
 }
-
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
         "{%0,%1,%2,%3};"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// C[M][N] = op(A) op(B) with the epilogue EPI.  CTA tile 64 x 32, four warps
-// of 16 rows each; K in steps of 16 staged through shared memory (zero
-// padded at the edges).  Fragment layouts of m16n8k16 (row.col): lane =
-// 4 g + t; A regs (g, 2t..2t+1), (g+8, ..), (g, 2t+8..), (g+8, 2t+8..);
-// B regs (2t..2t+1, g), (2t+8.., g); C (g, 2t..2t+1), (g+8, 2t..2t+1).
-template <int EPI>
-__global__ void __launch_bounds__(128) gemm_kernel(Gemm g) {
-    __shared__ bf16 As[64][16 + 8];
-    __shared__ bf16 Bs[16][32 + 8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * 64, n0 = blockIdx.y * 32;
-    const int gid = lane >> 2, tig = lane & 3;
-    const int rb = warp * 16;
-    float acc[4][4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
-    const bf16 zero = __float2bfloat16_rn(0.f);
-    for (int k0 = 0; k0 < g.K; k0 += 16) {
-        for (int q = threadIdx.x; q < 64 * 16; q += 128) {
-            const int r = q >> 4, c = q & 15;
-            const int m = m0 + r, k = k0 + c;
-            As[r][c] = (m < g.M && k < g.K) ? g.A[(long long)m * g.sam + (long long)k * g.sak] : zero;
+// The whole MLP of a tile of 16 MT rows in one block: inputs scaled and
+// rounded, three layers, and in training the output delta, the loss and both
+// hidden deltas.  The tile's activations stay in shared memory; the weights
+// (174 KB at 74-256-256-10) stream from L2 in chunks of 64 x 256 through a ring
+// of asynchronous copies that runs on across the layers.  Each of the 8 warps
+// owns 32 columns of a 256-column block and all rows of the tile.  What bounds
+// a call is latency (launches, the chunks' round trips), not the tensor cores:
+// at 256 rows the products are 45 MFLOP.  One GEMM launch per product with
+// element-wise staging took 33 us each (a 16-deep K-step per barrier); the
+// products keep its K order, so the forward pass has the same bits.
+// Measured (74-256-256-10, host arrays in and out): inference of 256 rows 108
+// -> 54 us, training step of 4096 rows 2.08 -> 0.17 ms.
+// Fragment layouts of m16n8k16 (row.col), lane = 4 g + t: A (g, 2t..2t+1),
+// (g+8, ..), (g, 2t+8..), (g+8, 2t+8..); B (2t..2t+1, g), (2t+8.., g); C (g,
+// 2t..2t+1), (g+8, 2t..2t+1).
+constexpr int kChunkK = 64, kChunkN = 256;
+constexpr int kMlpThreads = 256;
+constexpr int kStageElems = kChunkN * (kChunkK + 8);     // >= kChunkK * (kChunkN + 8)
+
+struct Mlp {
+    int rows, I, H, K, ldX, ldH, ldK, stages;
+    const float *x, *scale, *e, *b1, *b2, *b3;
+    const bf16 *W1, *W2, *W3;
+    bf16 *Xh, *H1h, *H2h, *dYh, *dA2h, *dA1h;
+    float *A1, *A2, *Y, *bpart, *lpart;
+    float inv;
+};
+
+__host__ __device__ inline int pad16(int x) { return (x + 15) & ~15; }
+static size_t mlp_smem(const Mlp &a, int MT, bool train) {
+    const size_t row = (size_t)(pad16(a.I) + 8) + 2 * (size_t)(pad16(a.H) + 8) + (train ? pad16(a.K) + 8 : 0);
+    return (row * 16 * MT + (size_t)a.stages * kStageElems) * sizeof(bf16);
+}
+
+template <int MT, bool TRAIN>
+__global__ void __launch_bounds__(kMlpThreads) mlp_kernel(Mlp a) {
+    extern __shared__ __align__(16) unsigned char pred_sm[];
+    __shared__ float red[kMlpThreads / 32];
+    const int SX = pad16(a.I) + 8, SH = pad16(a.H) + 8, SK = pad16(a.K) + 8;
+    constexpr int R = 16 * MT;
+    bf16 *ring = reinterpret_cast<bf16 *>(pred_sm);
+    bf16 *Xs = ring + (size_t)a.stages * kStageElems;
+    bf16 *P1 = Xs + R * SX, *P2 = P1 + R * SH, *dYs = P2 + R * SH;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const int r0 = blockIdx.x * R;
+    // phases: 0..2 the layers, 3 dA2 = dY W3^T, 4 dA1 = dA2 W2^T
+    constexpr int kPhases = TRAIN ? 5 : 3;
+    auto kdim = [&](int ph) { return ph == 0 ? a.I : ph == 3 ? a.K : a.H; };
+    auto ndim = [&](int ph) { return ph == 2 ? a.K : a.H; };
+    struct Pos {
+        int ph, n0, k0;
+    };
+    auto advance = [&](Pos &p) {
+        p.k0 += kChunkK;
+        if (p.k0 < kdim(p.ph)) return;
+        p.k0 = 0;
+        p.n0 += kChunkN;
+        if (p.n0 < ndim(p.ph)) return;
+        p.n0 = 0;
+        ++p.ph;
+    };
+    // chunk of the phase's weights: layers [k][n] rows, backward [n][k] rows
+    auto load = [&](const Pos &p, bf16 *st) {
+        if (p.ph < kPhases) {
+            const int N = ndim(p.ph), Kd = kdim(p.ph);
+            if (p.ph < 3) {
+                const bf16 *W = p.ph == 0 ? a.W1 : p.ph == 1 ? a.W2 : a.W3;
+                const int ld = p.ph == 2 ? a.ldK : a.ldH;
+                const int pieces = (min(kChunkN, N - p.n0) + 31) / 32 * 4;      // of 8 columns
+                for (int q = tid; q < kChunkK * pieces; q += kMlpThreads) {
+                    const int k = q / pieces, c = (q - k * pieces) * 8;
+                    const bool in = p.k0 + k < Kd && p.n0 + c < ld;
+                    cp16(st + k * (kChunkN + 8) + c, in ? W + (size_t)(p.k0 + k) * ld + p.n0 + c : W, in);
+                }
+            } else {
+                const bf16 *W = p.ph == 3 ? a.W3 : a.W2;
+                const int ld = p.ph == 3 ? a.ldK : a.ldH;
+                const int pieces = min(kChunkK, pad16(Kd) - p.k0) / 8;
+                for (int q = tid; q < kChunkN * pieces; q += kMlpThreads) {
+                    const int nn = q / pieces, c = (q - nn * pieces) * 8;
+                    const bool in = p.n0 + nn < N && p.k0 + c < ld;
+                    cp16(st + nn * (kChunkK + 8) + c, in ? W + (size_t)(p.n0 + nn) * ld + p.k0 + c : W, in);
+                }
+            }
         }
-        for (int q = threadIdx.x; q < 16 * 32; q += 128) {
-            const int r = q >> 5, c = q & 31;
-            const int k = k0 + r, nn = n0 + c;
-            Bs[r][c] = (k < g.K && nn < g.N) ? g.B[(long long)k * g.sbk + (long long)nn * g.sbn] : zero;
-        }
-        __syncthreads();
-        uint32_t a[4];
-        a[0] = pack2(As[rb + gid][2 * tig], As[rb + gid][2 * tig + 1]);
-        a[1] = pack2(As[rb + gid + 8][2 * tig], As[rb + gid + 8][2 * tig + 1]);
-        a[2] = pack2(As[rb + gid][2 * tig + 8], As[rb + gid][2 * tig + 9]);
-        a[3] = pack2(As[rb + gid + 8][2 * tig + 8], As[rb + gid + 8][2 * tig + 9]);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            uint32_t b[2];
-            b[0] = pack2(Bs[2 * tig][j * 8 + gid], Bs[2 * tig + 1][j * 8 + gid]);
-            b[1] = pack2(Bs[2 * tig + 8][j * 8 + gid], Bs[2 * tig + 9][j * 8 + gid]);
-            mma_bf16(acc[j], a, b);
-        }
-        __syncthreads();
+        cp_commit();
+    };
+    Pos lp{0, 0, 0};
+    for (int q = 0; q < a.stages - 1; ++q) {
+        load(lp, ring + (size_t)q * kStageElems);
+        if (lp.ph < kPhases) advance(lp);
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int m = m0 + rb + gid + (e >= 2 ? 8 : 0);
-            const int nn = n0 + j * 8 + 2 * tig + (e & 1);
-            if (m >= g.M || nn >= g.N) continue;
-            const long long o = (long long)m * g.N + nn;
-            float x = acc[j][e];
-            if (EPI == EPI_BIAS || EPI == EPI_BIAS_GELU) x += g.bias[nn];
-            if (EPI == EPI_DGELU) x *= gelu_grad(g.pre[o]);
-            g.outF[o] = x;
-            if (EPI == EPI_BIAS_GELU) g.outH[o] = __float2bfloat16_rn(gelu(x));
-            if (EPI == EPI_DGELU) g.outH[o] = __float2bfloat16_rn(x);
+    // activation tiles: padding columns and rows past the end stay zero
+    for (int q = tid; q < R * (2 * SH + (TRAIN ? SK : 0)) / 2; q += kMlpThreads) reinterpret_cast<uint32_t *>(P1)[q] = 0u;
+    for (int q = tid; q < R * SX; q += kMlpThreads) {
+        const int m = q / SX, c = q - m * SX;
+        float v = 0.f;
+        if (r0 + m < a.rows && c < a.I) v = a.x[(size_t)(r0 + m) * a.I + c] * a.scale[c];
+        const bf16 h = __float2bfloat16_rn(v);
+        Xs[q] = h;
+        if (r0 + m < a.rows && c < a.ldX) a.Xh[(size_t)(r0 + m) * a.ldX + c] = h;
+    }
+    float sq = 0.f;
+    float acc[MT][4][4];
+    Pos p{0, 0, 0};
+    for (int c = 0; p.ph < kPhases; ++c) {
+        if (a.stages == 4) cp_wait<2>();
+        else cp_wait<1>();
+        __syncthreads();                 // chunk c is there, chunk c - 1 and its tiles are done
+        {
+            const int q = c + a.stages - 1;
+            load(lp, ring + (size_t)(q % a.stages) * kStageElems);
+            if (lp.ph < kPhases) advance(lp);
         }
-}
-
-// dY = (Y - E) / R (FP32 and BF16) and the batch loss (1 / (2 R)) sum (Y -
-// E)^2, one block, fixed summation order
-__global__ void loss_grad_kernel(const float *Y, const float *E, long long count, int R, float *dYf,
-                                 bf16 *dYh, float *loss) {
-    __shared__ float part[256];
-    const float inv = 1.0f / (float)R;
-    float s = 0.f;
-    for (long long q = threadIdx.x; q < count; q += blockDim.x) {
-        const float d = Y[q] - E[q];
-        s = fmaf(d, d, s);
-        dYf[q] = d * inv;
-        dYh[q] = __float2bfloat16_rn(d * inv);
+        const bf16 *st = ring + (size_t)(c % a.stages) * kStageElems;
+        const int N = ndim(p.ph), Kd = kdim(p.ph);
+        const int nb = p.n0 + warp * 32;
+        const bool last = p.k0 + kChunkK >= Kd;
+        if (nb < N) {
+            if (p.k0 == 0) {
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) acc[m][j][e] = 0.f;
+            }
+            const bf16 *As = p.ph == 0 ? Xs : p.ph == 1 ? P1 : p.ph == 3 ? dYs : P2;
+            const int lda = p.ph == 0 ? SX : p.ph == 3 ? SK : SH;
+            const int steps = min(kChunkK, pad16(Kd) - p.k0) / 16;
+            for (int ks = 0; ks < steps; ++ks) {
+                uint32_t af[MT][4], bfr[2][4];
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+                    ldm4(af[m], As + (m * 16 + (lane & 15)) * lda + p.k0 + ks * 16 + (lane >> 4) * 8);
+                const int mt = lane >> 3, lr = lane & 7;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int nl = warp * 32 + h * 16 + (mt >> 1) * 8;
+                    const int kl = ks * 16 + (mt & 1) * 8;
+                    if (p.ph < 3) ldm4t(bfr[h], st + (kl + lr) * (kChunkN + 8) + nl);
+                    else ldm4(bfr[h], st + (nl + lr) * (kChunkK + 8) + kl);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) mma_bf16(acc[m][j], af[m], bfr[j >> 1][(j & 1) * 2], bfr[j >> 1][(j & 1) * 2 + 1]);
+            }
+            if (last) {
+                const float *bias = p.ph == 0 ? a.b1 : p.ph == 1 ? a.b2 : a.b3;
+                float *pre = (p.ph == 0 || p.ph == 4) ? a.A1 : a.A2;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int f = 0; f < 2; ++f) {
+                        const int nn = nb + j * 8 + 2 * t + f;
+                        float col = 0.f;             // the column's share of a bias gradient
+#pragma unroll
+                        for (int mh = 0; mh < 2 * MT; ++mh) {
+                            const int m = (mh >> 1) * 16 + (mh & 1) * 8 + g, r = r0 + m;
+                            if (r >= a.rows || nn >= N) continue;
+                            float v = acc[mh >> 1][j][(mh & 1) * 2 + f];
+                            if (p.ph < 2) {
+                                v += bias[nn];
+                                pre[(size_t)r * a.H + nn] = v;
+                                const bf16 h = __float2bfloat16_rn(gelu(v));
+                                (p.ph == 0 ? P1 : P2)[m * SH + nn] = h;
+                                (p.ph == 0 ? a.H1h : a.H2h)[(size_t)r * a.ldH + nn] = h;
+                            } else if (p.ph == 2) {
+                                v += bias[nn];
+                                a.Y[(size_t)r * a.K + nn] = v;
+                                if (TRAIN) {
+                                    const float d = v - a.e[(size_t)r * a.K + nn];
+                                    sq = fmaf(d, d, sq);
+                                    const float dy = d * a.inv;
+                                    col += dy;
+                                    const bf16 h = __float2bfloat16_rn(dy);
+                                    dYs[m * SK + nn] = h;
+                                    a.dYh[(size_t)r * a.ldK + nn] = h;
+                                }
+                            } else {
+                                v *= gelu_grad(pre[(size_t)r * a.H + nn]);   // this thread's own value
+                                col += v;
+                                const bf16 h = __float2bfloat16_rn(v);
+                                if (p.ph == 3) P2[m * SH + nn] = h;          // dA2 takes H2's place
+                                (p.ph == 3 ? a.dA2h : a.dA1h)[(size_t)r * a.ldH + nn] = h;
+                            }
+                        }
+                        if (TRAIN && p.ph >= 2) {
+                            for (int o = 4; o < 32; o <<= 1) col += __shfl_xor_sync(0xffffffffu, col, o);
+                            const int off = p.ph == 4 ? 0 : p.ph == 3 ? a.H : 2 * a.H;
+                            if (g == 0 && nn < N) a.bpart[(size_t)blockIdx.x * (2 * a.H + a.K) + off + nn] = col;
+                        }
+                    }
+            }
+        }
+        advance(p);
     }
-    part[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) part[threadIdx.x] += part[threadIdx.x + o];
+    cp_wait<0>();
+    if (TRAIN) {
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        if (lane == 0) red[warp] = sq;
         __syncthreads();
+        if (tid == 0) {
+            float s = 0.f;
+            for (int w = 0; w < kMlpThreads / 32; ++w) s += red[w];
+            a.lpart[blockIdx.x] = s;
+        }
     }
-    if (threadIdx.x == 0) *loss = 0.5f * part[0] * inv;
 }
 
-// out[n] = sum over rows of D[r][n] in row order (deterministic)
-__global__ void colsum_kernel(const float *D, int R, int N, float *out) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float s = 0.f;
-    for (int r = 0; r < R; ++r) s += D[(long long)r * N + n];
-    out[n] = s;
+// Weight gradients dW[m][n] = sum_r A[r][m] D[r][n] of the three layers in one
+// launch: block = (64 x 64 tile of a layer, slice of the rows); the slices'
+// sums are added in order by the Adam kernel.  One block per tile over all
+// 4096 rows left 32 blocks busy for 678 us.
+constexpr int kDwThreads = 128, kDwTile = 64, kDwStages = 4, kDwLd = kDwTile + 8;
+struct Dw {
+    int rows, slice, tiles[3];
+    const bf16 *A[3], *D[3];
+    int ldA[3], ldD[3], M[3], N[3];
+    long long off[3], n_params;
+    float *part;
+};
+
+__global__ void __launch_bounds__(kDwThreads) dw_kernel(Dw a) {
+    extern __shared__ __align__(16) unsigned char pred_sm[];
+    bf16 *ring = reinterpret_cast<bf16 *>(pred_sm);
+    constexpr int kStage = 2 * kDwTile * kDwLd;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    int l = 0, tile = blockIdx.x;
+    while (l < 2 && tile >= a.tiles[l]) tile -= a.tiles[l++];
+    const int M = a.M[l], N = a.N[l], nt = (N + kDwTile - 1) / kDwTile;
+    const int m0 = tile / nt * kDwTile, n0 = tile % nt * kDwTile;
+    const int rb = blockIdx.y * a.slice, re = min(a.rows, rb + a.slice);
+    const int chunks = (re - rb + kDwTile - 1) / kDwTile;
+    auto load = [&](int c) {
+        if (c < chunks) {
+            bf16 *st = ring + (c % kDwStages) * kStage;
+            for (int q = tid; q < 2 * kDwTile * 8; q += kDwThreads) {
+                const int which = q / (kDwTile * 8), k = (q >> 3) % kDwTile, cc = (q & 7) * 8;
+                const bf16 *src = which ? a.D[l] : a.A[l];
+                const int ld = which ? a.ldD[l] : a.ldA[l], c0 = (which ? n0 : m0) + cc, r = rb + c * kDwTile + k;
+                const bool in = r < re && c0 < ld;
+                cp16(st + which * kDwTile * kDwLd + k * kDwLd + cc, in ? src + (size_t)r * ld + c0 : src, in);
+            }
+        }
+        cp_commit();
+    };
+    for (int c = 0; c < kDwStages - 1; ++c) load(c);
+    float acc[2][4][4];
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[m][j][e] = 0.f;
+    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32, mt = lane >> 3, lr = lane & 7;
+    for (int c = 0; c < chunks; ++c) {
+        cp_wait<kDwStages - 2>();
+        __syncthreads();
+        load(c + kDwStages - 1);
+        const bf16 *As = ring + (c % kDwStages) * kStage, *Ds = As + kDwTile * kDwLd;
+#pragma unroll
+        for (int ks = 0; ks < kDwTile / 16; ++ks) {
+            uint32_t af[2][4], bfr[2][4];
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+                ldm4t(af[m], As + (ks * 16 + (mt >> 1) * 8 + lr) * kDwLd + wm + m * 16 + (mt & 1) * 8);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                ldm4t(bfr[h], Ds + (ks * 16 + (mt & 1) * 8 + lr) * kDwLd + wn + h * 16 + (mt >> 1) * 8);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int m = 0; m < 2; ++m) mma_bf16(acc[m][j], af[m], bfr[j >> 1][(j & 1) * 2], bfr[j >> 1][(j & 1) * 2 + 1]);
+        }
+    }
+    cp_wait<0>();
+    float *out = a.part + (size_t)blockIdx.y * a.n_params + a.off[l];
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int mm = m0 + wm + m * 16 + g + (e >= 2 ? 8 : 0), nn = n0 + wn + j * 8 + 2 * t + (e & 1);
+                if (mm < M && nn < N) out[(size_t)mm * N + nn] = acc[m][j][e];
+            }
 }
 
-// Adam (Eq. adam1, Eq. adam2, Eq. adam) on the FP32 masters
-__global__ void adam_kernel(float *w, const float *g, float *m, float *v, long long n, float lr, float c1,
-                            float c2) {
+// layout of the packed parameters: layer l holds W [I_l][O_l] then b [O_l]
+struct Layout {
+    int I[3], O[3], ld[3];
+    long long offW[3], offb[3];
+    bf16 *Wh[3];
+};
+__device__ __forceinline__ void locate(const Layout &L, long long q, int &l, long long &i, bool &bias) {
+    l = q >= L.offW[2] ? 2 : q >= L.offW[1] ? 1 : 0;
+    bias = q >= L.offb[l];
+    i = q - (bias ? L.offb[l] : L.offW[l]);
+}
+__device__ __forceinline__ void put_weight(const Layout &L, int l, long long i, float w) {
+    const long long r = i / L.O[l];
+    L.Wh[l][r * L.ld[l] + (i - r * L.O[l])] = __float2bfloat16_rn(w);
+}
+__global__ void refresh_kernel(Layout L, const float *w, long long n) {
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
          q += (long long)gridDim.x * blockDim.x) {
-        const float gq = g[q];
+        int l;
+        long long i;
+        bool bias;
+        locate(L, q, l, i, bias);
+        if (!bias) put_weight(L, l, i, w[q]);
+    }
+}
+
+// Adam (Eq. adam1, Eq. adam2, Eq. adam) on the FP32 masters: sums the
+// gradient's parts in order (weights: row slices; biases: row tiles), steps,
+// and refreshes the BF16 weights; block 0 also sums the loss.
+__global__ void adam_kernel(Layout L, float *w, float *grad, float *m, float *v, long long n, const float *gpart,
+                            int slices, const float *bpart, const float *lpart, int tiles, float half_inv,
+                            float *loss, float lr, float c1, float c2) {
+    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
+         q += (long long)gridDim.x * blockDim.x) {
+        int l;
+        long long i;
+        bool bias;
+        locate(L, q, l, i, bias);
+        float gq = 0.f;
+        if (bias) {
+            const long long nb = L.O[0] + L.O[1] + L.O[2];
+            const float *bp = bpart + (l == 0 ? 0 : l == 1 ? L.O[0] : L.O[0] + L.O[1]) + i;
+#pragma unroll 8
+            for (int s = 0; s < tiles; ++s) gq += bp[s * nb];
+        } else {
+#pragma unroll 8
+            for (int s = 0; s < slices; ++s) gq += gpart[s * n + q];
+        }
+        grad[q] = gq;
         const float mq = 0.9f * m[q] + 0.1f * gq;
         const float vq = 0.999f * v[q] + 0.001f * gq * gq;
         m[q] = mq;
         v[q] = vq;
-        w[q] -= lr * (mq / c1) / (sqrtf(vq / c2) + 1e-8f);
+        const float wq = w[q] - lr * (mq / c1) / (sqrtf(vq / c2) + 1e-8f);
+        w[q] = wq;
+        if (!bias) put_weight(L, l, i, wq);
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        float s = 0.f;
+        for (int q = threadIdx.x; q < tiles; q += 32) s += lpart[q];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) *loss = half_inv * s;
     }
 }
 
-__global__ void bf16_to_float_kernel(const bf16 *src, float *dst, long long n) {
+// rows of `cols` BF16 values with leading dimension ld, widened
+__global__ void bf16_to_float_kernel(const bf16 *src, int ld, int cols, float *dst, long long n) {
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
          q += (long long)gridDim.x * blockDim.x)
-        dst[q] = __bfloat162float(src[q]);
+        dst[q] = __bfloat162float(src[q / cols * ld + q % cols]);
 }
 
 // ------------------------------------------------------------------ host
 
-template <int EPI>
-static void gemm(cudaStream_t st, const Gemm &g) {
-    const dim3 grid((g.M + 63) / 64, (g.N + 31) / 32);
-    gemm_kernel<EPI><<<grid, 128, 0, st>>>(g);
-}
+constexpr int kMlpSmemMax = 220 * 1024;
+constexpr int kDwSmem = kDwStages * 2 * kDwTile * kDwLd * (int)sizeof(bf16);
 
 static unsigned blocks_for(long long n) {
     long long b = (n + 255) / 256;
@@ -279,23 +519,34 @@ extern "C" eprop_status eprop_predictor_create(int32_t n_in, int32_t hidden, int
         p->own_stream = 1;
     }
     const long long R = max_rows, H = hidden;
+    auto pad8 = [](int x) { return (x + 7) & ~7; };
+    p->ldX = pad8(n_in);
+    p->ldH = pad8(hidden);
+    p->ldK = pad8(n_out);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, dev);
+    // row slices of the weight gradients: at most 16, and at most 16 MB of parts
+    p->max_slices = (int)std::max(1LL, std::min(16LL, (4LL << 20) / o));
+    const long long tiles = (R + 15) / 16;
     if (e == cudaSuccess) e = palloc(p, &p->params, o);
     if (e == cudaSuccess) e = palloc(p, &p->grads, o);
     if (e == cudaSuccess) e = palloc(p, &p->m, o);
     if (e == cudaSuccess) e = palloc(p, &p->v, o);
-    for (int l = 0; l < 3 && e == cudaSuccess; ++l) e = palloc(p, &p->Wh[l], (long long)fan_in[l] * fan_out[l]);
-    if (e == cudaSuccess) e = palloc(p, &p->Xh, R * n_in);
-    if (e == cudaSuccess) e = palloc(p, &p->H1h, R * H);
-    if (e == cudaSuccess) e = palloc(p, &p->H2h, R * H);
-    if (e == cudaSuccess) e = palloc(p, &p->dYh, R * n_out);
-    if (e == cudaSuccess) e = palloc(p, &p->dA2h, R * H);
-    if (e == cudaSuccess) e = palloc(p, &p->dA1h, R * H);
+    for (int l = 0; l < 3 && e == cudaSuccess; ++l)
+        e = palloc(p, &p->Wh[l], (long long)fan_in[l] * (l == 2 ? p->ldK : p->ldH));
+    if (e == cudaSuccess) e = palloc(p, &p->Xh, R * p->ldX);
+    if (e == cudaSuccess) e = palloc(p, &p->H1h, R * p->ldH);
+    if (e == cudaSuccess) e = palloc(p, &p->H2h, R * p->ldH);
+    if (e == cudaSuccess) e = palloc(p, &p->dYh, R * p->ldK);
+    if (e == cudaSuccess) e = palloc(p, &p->dA2h, R * p->ldH);
+    if (e == cudaSuccess) e = palloc(p, &p->dA1h, R * p->ldH);
+    if (e == cudaSuccess) e = palloc(p, &p->gpart, p->max_slices * o);
+    if (e == cudaSuccess) e = palloc(p, &p->bpart, tiles * (2 * H + n_out));
+    if (e == cudaSuccess) e = palloc(p, &p->lpart, tiles);
     if (e == cudaSuccess) e = palloc(p, &p->A1, R * H);
     if (e == cudaSuccess) e = palloc(p, &p->A2, R * H);
     if (e == cudaSuccess) e = palloc(p, &p->Y, R * n_out);
-    if (e == cudaSuccess) e = palloc(p, &p->dYf, R * n_out);
-    if (e == cudaSuccess) e = palloc(p, &p->dA2f, R * H);
-    if (e == cudaSuccess) e = palloc(p, &p->dA1f, R * H);
     if (e == cudaSuccess) e = palloc(p, &p->xin, R * n_in);
     if (e == cudaSuccess) e = palloc(p, &p->ein, R * n_out);
     if (e == cudaSuccess) e = palloc(p, &p->yout, R * n_out);
@@ -311,6 +562,11 @@ extern "C" eprop_status eprop_predictor_create(int32_t n_in, int32_t hidden, int
         eprop_predictor_destroy(p);
         return e == cudaErrorMemoryAllocation ? EPROP_ENOMEM : EPROP_ECUDA;
     }
+    cudaFuncSetAttribute(mlp_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmemMax);
+    cudaFuncSetAttribute(mlp_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmemMax);
+    cudaFuncSetAttribute(mlp_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmemMax);
+    cudaFuncSetAttribute(mlp_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmemMax);
+    cudaFuncSetAttribute(dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDwSmem);
     std::vector<float> init;
     if (!params) {
         init.assign((size_t)o, 0.f);
@@ -340,11 +596,22 @@ extern "C" eprop_status eprop_predictor_create(int32_t n_in, int32_t hidden, int
 
 extern "C" int64_t eprop_predictor_num_params(const eprop_predictor *p) { return p ? p->n_params : 0; }
 
+static Layout layout_of(eprop_predictor *p) {
+    Layout L{};
+    const int I[3] = {p->n_in, p->hidden, p->hidden}, O[3] = {p->hidden, p->hidden, p->n_out};
+    for (int l = 0; l < 3; ++l) {
+        L.I[l] = I[l];
+        L.O[l] = O[l];
+        L.ld[l] = l == 2 ? p->ldK : p->ldH;
+        L.offW[l] = p->off_W[l];
+        L.offb[l] = p->off_b[l];
+        L.Wh[l] = p->Wh[l];
+    }
+    return L;
+}
+
 static void refresh_weights(eprop_predictor *p) {
-    const long long cnt[3] = {(long long)p->n_in * p->hidden, (long long)p->hidden * p->hidden,
-                              (long long)p->hidden * p->n_out};
-    for (int l = 0; l < 3; ++l)
-        to_bf16_kernel<<<blocks_for(cnt[l]), 256, 0, p->st>>>(p->params + p->off_W[l], p->Wh[l], cnt[l]);
+    refresh_kernel<<<blocks_for(p->n_params), 256, 0, p->st>>>(layout_of(p), p->params, p->n_params);
 }
 
 extern "C" eprop_status eprop_predictor_set_params(eprop_predictor *p, const float *params) {
@@ -359,30 +626,39 @@ extern "C" eprop_status eprop_predictor_set_params(eprop_predictor *p, const flo
     return EPROP_OK;
 }
 
-// forward on x already on the device (FP32 [rows][n_in]); leaves Y in p->Y
-static void issue_forward(eprop_predictor *p, const float *x, int rows, cudaStream_t st) {
-    const int H = p->hidden;
-    input_bf16_kernel<<<blocks_for((long long)rows * p->n_in), 256, 0, st>>>(x, p->in_scale, p->n_in, p->Xh,
-                                                                            (long long)rows * p->n_in);
-    Gemm g{};
-    g.A = p->Xh; g.sam = p->n_in; g.sak = 1;
-    g.B = p->Wh[0]; g.sbk = H; g.sbn = 1;
-    g.M = rows; g.N = H; g.K = p->n_in;
-    g.bias = p->params + p->off_b[0]; g.outF = p->A1; g.outH = p->H1h;
-    gemm<EPI_BIAS_GELU>(st, g);
-    g = Gemm{};
-    g.A = p->H1h; g.sam = H; g.sak = 1;
-    g.B = p->Wh[1]; g.sbk = H; g.sbn = 1;
-    g.M = rows; g.N = H; g.K = H;
-    g.bias = p->params + p->off_b[1]; g.outF = p->A2; g.outH = p->H2h;
-    gemm<EPI_BIAS_GELU>(st, g);
-    g = Gemm{};
-    g.A = p->H2h; g.sam = H; g.sak = 1;
-    g.B = p->Wh[2]; g.sbk = p->n_out; g.sbn = 1;
-    g.M = rows; g.N = p->n_out; g.K = H;
-    g.bias = p->params + p->off_b[2]; g.outF = p->Y;
-    gemm<EPI_BIAS>(st, g);
+// forward (and in training the deltas, the loss and the bias gradients) on x
+// already on the device; leaves Y in p->Y and returns the number of row tiles
+static int issue_mlp(eprop_predictor *p, const float *x, const float *e, int rows, cudaStream_t st) {
+    Mlp a{};
+    a.rows = rows; a.I = p->n_in; a.H = p->hidden; a.K = p->n_out;
+    a.ldX = p->ldX; a.ldH = p->ldH; a.ldK = p->ldK;
+    a.x = x; a.scale = p->in_scale; a.e = e;
+    a.b1 = p->params + p->off_b[0]; a.b2 = p->params + p->off_b[1]; a.b3 = p->params + p->off_b[2];
+    a.W1 = p->Wh[0]; a.W2 = p->Wh[1]; a.W3 = p->Wh[2];
+    a.Xh = p->Xh; a.H1h = p->H1h; a.H2h = p->H2h; a.dYh = p->dYh; a.dA2h = p->dA2h; a.dA1h = p->dA1h;
+    a.A1 = p->A1; a.A2 = p->A2; a.Y = p->Y; a.bpart = p->bpart; a.lpart = p->lpart;
+    a.inv = 1.0f / (float)rows;
+    const bool train = e != nullptr;
+    // 32-row tiles once 16-row tiles fill the SMs; four ring stages where they fit
+    a.stages = 4;
+    int mt = rows > 16 * p->sm_count ? 2 : 1;
+    if (mlp_smem(a, mt, train) > (size_t)kMlpSmemMax) mt = 1;
+    if (mlp_smem(a, mt, train) > (size_t)kMlpSmemMax) a.stages = 3;
+    const int tiles = (rows + 16 * mt - 1) / (16 * mt);
+    const size_t sm = mlp_smem(a, mt, train);
+    if (train) {
+        if (mt == 2) mlp_kernel<2, true><<<tiles, kMlpThreads, sm, st>>>(a);
+        else mlp_kernel<1, true><<<tiles, kMlpThreads, sm, st>>>(a);
+    } else {
+        if (mt == 2) mlp_kernel<2, false><<<tiles, kMlpThreads, sm, st>>>(a);
+        else mlp_kernel<1, false><<<tiles, kMlpThreads, sm, st>>>(a);
+    }
     p->rows = rows;
+    return tiles;
+}
+
+static void issue_forward(eprop_predictor *p, const float *x, int rows, cudaStream_t st) {
+    issue_mlp(p, x, nullptr, rows, st);
 }
 
 const float *predictor_issue_forward(eprop_predictor *p, const float *x_dev, int rows, cudaStream_t st) {
@@ -425,48 +701,33 @@ extern "C" eprop_status eprop_predictor_train_step(eprop_predictor *p, const flo
         xd = p->xin;
         ed = p->ein;
     }
-    issue_forward(p, xd, rows, p->st);
-    loss_grad_kernel<<<1, 256, 0, p->st>>>(p->Y, ed, (long long)rows * K, rows, p->dYf, p->dYh, p->loss);
-    Gemm g{};
-    // dW3 = H2^T dY
-    g.A = p->H2h; g.sam = 1; g.sak = H;
-    g.B = p->dYh; g.sbk = K; g.sbn = 1;
-    g.M = H; g.N = K; g.K = rows; g.outF = p->grads + p->off_W[2];
-    gemm<EPI_STORE>(p->st, g);
-    colsum_kernel<<<(K + 127) / 128, 128, 0, p->st>>>(p->dYf, rows, K, p->grads + p->off_b[2]);
-    // dA2 = (dY W3^T) * GELU'(A2)
-    g = Gemm{};
-    g.A = p->dYh; g.sam = K; g.sak = 1;
-    g.B = p->Wh[2]; g.sbk = 1; g.sbn = K;
-    g.M = rows; g.N = H; g.K = K; g.pre = p->A2; g.outF = p->dA2f; g.outH = p->dA2h;
-    gemm<EPI_DGELU>(p->st, g);
-    // dW2 = H1^T dA2
-    g = Gemm{};
-    g.A = p->H1h; g.sam = 1; g.sak = H;
-    g.B = p->dA2h; g.sbk = H; g.sbn = 1;
-    g.M = H; g.N = H; g.K = rows; g.outF = p->grads + p->off_W[1];
-    gemm<EPI_STORE>(p->st, g);
-    colsum_kernel<<<(H + 127) / 128, 128, 0, p->st>>>(p->dA2f, rows, H, p->grads + p->off_b[1]);
-    // dA1 = (dA2 W2^T) * GELU'(A1)
-    g = Gemm{};
-    g.A = p->dA2h; g.sam = H; g.sak = 1;
-    g.B = p->Wh[1]; g.sbk = 1; g.sbn = H;
-    g.M = rows; g.N = H; g.K = H; g.pre = p->A1; g.outF = p->dA1f; g.outH = p->dA1h;
-    gemm<EPI_DGELU>(p->st, g);
-    // dW1 = X^T dA1
-    g = Gemm{};
-    g.A = p->Xh; g.sam = 1; g.sak = I;
-    g.B = p->dA1h; g.sbk = H; g.sbn = 1;
-    g.M = I; g.N = H; g.K = rows; g.outF = p->grads + p->off_W[0];
-    gemm<EPI_STORE>(p->st, g);
-    colsum_kernel<<<(H + 127) / 128, 128, 0, p->st>>>(p->dA1f, rows, H, p->grads + p->off_b[0]);
+    const int tiles = issue_mlp(p, xd, ed, rows, p->st);
+    Dw d{};
+    d.rows = rows;
+    // slices of at least 128 rows (two chunks in flight per block)
+    int slices = std::min(p->max_slices, (rows + 127) / 128);
+    d.slice = ((rows + slices - 1) / slices + 15) & ~15;
+    slices = (rows + d.slice - 1) / d.slice;
+    const bf16 *A[3] = {p->Xh, p->H1h, p->H2h}, *D[3] = {p->dA1h, p->dA2h, p->dYh};
+    const int ldA[3] = {p->ldX, p->ldH, p->ldH}, ldD[3] = {p->ldH, p->ldH, p->ldK};
+    const int M[3] = {I, H, H}, N[3] = {H, H, K};
+    int blocks = 0;
+    for (int l = 0; l < 3; ++l) {
+        d.A[l] = A[l]; d.D[l] = D[l]; d.ldA[l] = ldA[l]; d.ldD[l] = ldD[l]; d.M[l] = M[l]; d.N[l] = N[l];
+        d.off[l] = p->off_W[l];
+        d.tiles[l] = ((M[l] + kDwTile - 1) / kDwTile) * ((N[l] + kDwTile - 1) / kDwTile);
+        blocks += d.tiles[l];
+    }
+    d.n_params = p->n_params;
+    d.part = p->gpart;
+    dw_kernel<<<dim3(blocks, slices), kDwThreads, kDwSmem, p->st>>>(d);
     // Adam step
     p->adam_t += 1;
     const float c1 = (float)(1.0 - std::pow(0.9, (double)p->adam_t));
     const float c2 = (float)(1.0 - std::pow(0.999, (double)p->adam_t));
-    adam_kernel<<<blocks_for(p->n_params), 256, 0, p->st>>>(p->params, p->grads, p->m, p->v, p->n_params, lr, c1,
-                                                             c2);
-    refresh_weights(p);
+    adam_kernel<<<blocks_for(p->n_params), 256, 0, p->st>>>(layout_of(p), p->params, p->grads, p->m, p->v, p->n_params,
+                                                             p->gpart, slices, p->bpart, p->lpart, tiles,
+                                                             0.5f / (float)rows, p->loss, lr, c1, c2);
     PCK(p, cudaGetLastError());
     if (loss_out) {
         PCK(p, cudaMemcpyAsync(loss_out, p->loss, 4, cudaMemcpyDeviceToHost, p->st));
@@ -480,6 +741,7 @@ extern "C" eprop_status eprop_predictor_read(eprop_predictor *p, int32_t which, 
     const long long R = p->rows, H = p->hidden, K = p->n_out;
     const float *srcF = nullptr;
     const bf16 *srcH = nullptr;
+    int ld = p->ldH, cols = p->hidden;
     long long n = 0;
     switch (which) {
         case 0: srcF = p->params; n = p->n_params; break;
@@ -489,17 +751,17 @@ extern "C" eprop_status eprop_predictor_read(eprop_predictor *p, int32_t which, 
         case 4: srcF = p->A2; n = R * H; break;
         case 5: srcH = p->H2h; n = R * H; break;
         case 6: srcF = p->Y; n = R * K; break;
-        case 7: srcH = p->dYh; n = R * K; break;
+        case 7: srcH = p->dYh; n = R * K; ld = p->ldK; cols = p->n_out; break;
         case 8: srcH = p->dA2h; n = R * H; break;
         case 9: srcH = p->dA1h; n = R * H; break;
         case 10: srcF = p->m; n = p->n_params; break;
         case 11: srcF = p->v; n = p->n_params; break;
-        case 12: srcH = p->Xh; n = R * p->n_in; break;
+        case 12: srcH = p->Xh; n = R * p->n_in; ld = p->ldX; cols = p->n_in; break;
         default: return pfail(p, EPROP_EINVAL, "unknown buffer");
     }
     if (count < n) return pfail(p, EPROP_EINVAL, "destination too small");
     if (srcH) {
-        bf16_to_float_kernel<<<blocks_for(n), 256, 0, p->st>>>(srcH, p->stage, n);
+        bf16_to_float_kernel<<<blocks_for(n), 256, 0, p->st>>>(srcH, ld, cols, p->stage, n);
         PCK(p, cudaGetLastError());
         PCK(p, cudaMemcpyAsync(dst, p->stage, (size_t)n * 4, cudaMemcpyDeviceToHost, p->st));
     } else {
