@@ -817,8 +817,7 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
         if (persistent || sample_loop) {
             if (i % U != 0) continue;
         } else {
-        if (c.n_in > 0) { eprop::launch_inject(n, i, (int)net->max_in_per_step, st); L += 1; }
-        eprop::launch_neuron(n, i, net->sm_count, st);
+        eprop::launch_neuron(n, i, (int)net->max_in_per_step, st);
         fork_readout();
         eprop::launch_readout(n, i, net->sm_count, sr);
         if (n.pred_mode) {

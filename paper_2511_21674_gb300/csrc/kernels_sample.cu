@@ -201,7 +201,8 @@ __global__ void __launch_bounds__(BT, 1) sample_steps_kernel(Net n, int i0, int 
                         ring_hi[so + j] = 0u;
                         const int fz = n.forced ? (n.forced[((long long)b * T + (i - 1)) * N + j] ? 1 : 0) : -1;
                         float psi;
-                        neuron_core<VAR>(n, b, j, ck.t_abs_base + i, thr_s, acc, fz, st[q], psi, z);
+                        neuron_core<VAR>(n, j, ck.t_abs_base + i, drive_count(n, b, j, ck.t_abs_base + i, thr_s), acc, fz,
+                                         st[q], psi, z);
                         *psi_p[q] = psi;
                         psi_p[q] += N;
                         if (VAR && n.R_win) n.R_win[((long long)b * U + (i - i0)) * N + j] = rate_signal(n, st[q].rate);

@@ -15,25 +15,32 @@ struct NeuronRegs {
     float rate;
 };
 
-// Update of neuron j of sample b at absolute step t_abs from its arrivals
-// acc_q (fixed point) (Eq. lif_update, Eq. binary-spike-state-variable, Eq.
+// External drive of neuron j of sample b at absolute step t_abs: the number
+// of thresholds at or below the hash's upper 32 bits (0 without drive).
+__device__ __forceinline__ int drive_count(const Net &n, int b, int j, long long t_abs, const uint32_t *thr_s) {
+    if (n.n_thr == 0) return 0;
+    const uint64_t h = mix64(mix64(mix64(n.drive_seed ^ (uint64_t)j) ^ (uint64_t)t_abs) ^ (uint64_t)b);
+    const uint32_t u = (uint32_t)(h >> 32);
+    // thresholds are non-decreasing (checked at creation): the count of
+    // thresholds <= u is the index of the first one above u
+    int cnt = 0;
+    while (cnt < n.n_thr && u >= thr_s[cnt]) ++cnt;
+    return cnt;
+}
+
+// Update of neuron j at absolute step t_abs from its arrivals acc_q (fixed
+// point) and its drive count (Eq. lif_update, Eq. binary-spike-state-variable, Eq.
 // spike-threshold-adaptation, the surrogate).  forced_z >= 0 gives the spike.
 // VAR: the e-prop+ variants (fixed reset, ignore-and-fire, exponential
 // surrogate, rate regularisation) are compiled in; the plain method's
 // instance carries none of their code.
 template <bool VAR>
-__device__ __forceinline__ void neuron_core(const Net &n, int b, int j, long long t_abs, const uint32_t *thr_s,
-                                            long long acc_q, int forced_z, NeuronRegs &s, float &psi, int &z) {
+__device__ __forceinline__ void neuron_core(const Net &n, int j, long long t_abs, int cnt, long long acc_q,
+                                            int forced_z, NeuronRegs &s, float &psi, int &z) {
     // exact fixed-point input split into an FP32 pair
     float u_hi, u_lo;
     fixed_to_pair(acc_q, u_hi, u_lo);
     if (n.n_thr > 0) {
-        const uint64_t h = mix64(mix64(mix64(n.drive_seed ^ (uint64_t)j) ^ (uint64_t)t_abs) ^ (uint64_t)b);
-        const uint32_t u = (uint32_t)(h >> 32);
-        // thresholds are non-decreasing (checked at creation): the count of
-        // thresholds <= u is the index of the first one above u
-        int cnt = 0;
-        while (cnt < n.n_thr && u >= thr_s[cnt]) ++cnt;
         const float dv = n.drive_weight * (float)cnt;
         const float de = fmaf(n.drive_weight, (float)cnt, -dv);
         float e;
