@@ -1001,48 +1001,74 @@ __global__ void __launch_bounds__(256, MODE == kPassIdle ? 3 : 2) window_pass_ke
                 if (live[u]) cf[u] = load_coef_dense<ALIF>(n, td[u] & 0xFFFFFFu);
                 if (c0[u] >= 0) t0[u] = load_table<ALIF>(n, qa + (long long)a1 * N + (td[u] & 0xFFFFFFu));
             }
+float G[kB];
+#pragma unroll
+            for (int u = 0; u < kB; ++u) {
+                G[u] = 0.f;
+                if (!live[u]) continue;
+                float zbar = zr[u];
+                apply_coef<ALIF>(n, cf[u], zbar, ep[u], eb[u], G[u]);
+                if (LISTS && c0[u] >= 0) {
+                    G[u] += t0[u].x;
+                    eb[u] += t0[u].y;
+                    if (ALIF) ep[u] += t0[u].z;
+                }
+            }
+            if (LISTS) {
+                if (listed) {
+                    // further arrivals, spike by spike: the entries of the
+                    // batch's synapses are loaded together (synapse by synapse,
+                    // each arrival of a row with several spikes paid its own
+                    // round trip)
+                    for (int cc = 1; cc < ns; ++cc) {
+                        const int s = sp[cc];
+                        float4 t[kB];
+                        bool on[kB];
+#pragma unroll
+                        for (int u = 0; u < kB; ++u) {
+                            const int a = s + (int)(td[u] >> 24);
+                            on[u] = c0[u] >= 0 && cc > c0[u] && a <= r_end;
+                            if (on[u]) t[u] = load_table<ALIF>(n, qa + (long long)a * N + (td[u] & 0xFFFFFFu));
+                        }
+#pragma unroll
+                        for (int u = 0; u < kB; ++u) {
+                            if (!on[u]) continue;
+                            G[u] += t[u].x;
+                            eb[u] += t[u].y;
+                            if (ALIF) ep[u] += t[u].z;
+                        }
+                    }
+                } else {
+                    // rows with more spikes than the cache holds
+#pragma unroll
+                    for (int u = 0; u < kB; ++u) {
+                        const int dl = (int)(td[u] >> 24);
+                        if (!live[u]) continue;
+                        float g = G[u], e1 = eb[u], e2 = ep[u];    // only these have addresses
+                        scan_arrivals<ALIF>(n, src_words_c(n, 0, d.src), max(d.row, a0 + 1 - dl), r_end - dl, dl,
+                                            qa + (td[u] & 0xFFFFFFu), g, e1, e2);
+                        G[u] = g;
+                        eb[u] = e1;
+                        ep[u] = e2;
+                    }
+                }
+            }
 #pragma unroll
             for (int u = 0; u < kB; ++u) {
                 if (!live[u]) continue;
                 const int idx = lane + 32 * (h + u);
-                const int j = (int)(td[u] & 0xFFFFFFu);
-                const int dl = (int)(td[u] >> 24);
-                float G = 0.f, zbar = zr[u], ebar = eb[u], epsa = ep[u];
-                apply_coef<ALIF>(n, cf[u], zbar, epsa, ebar, G);
-                if (LISTS) {
-                    if (listed) {
-                        if (c0[u] >= 0) {
-                            G += t0[u].x;
-                            ebar += t0[u].y;
-                            if (ALIF) epsa += t0[u].z;
-                        }
-                        // further arrivals (rows with more than one spike)
-                        for (int cc = (c0[u] >= 0 ? c0[u] + 1 : ns); cc < ns; ++cc) {
-                            const int a = sp[cc] + dl;
-                            if (a > r_end) break;
-                            const float4 t = load_table<ALIF>(n, qa + (long long)a * N + j);
-                            G += t.x;
-                            ebar += t.y;
-                            if (ALIF) epsa += t.z;
-                        }
-                    } else {
-                        // rows with more spikes than the cache holds
-                        scan_arrivals<ALIF>(n, src_words_c(n, 0, d.src), max(d.row, a0 + 1 - dl), r_end - dl, dl,
-                                            qa + j, G, ebar, epsa);
-                    }
-                }
-                if (G != 0.f) {
+                if (G[u] != 0.f) {
                     if (GEN) {
-                        const float wn = window_update(n, d.q0 + idx, wv[u], G);
+                        const float wn = window_update(n, d.q0 + idx, wv[u], G[u]);
                         if (!n.adam) __stcs(wq + idx, wn);
                     } else {
-                        __stcs(wq + idx, sgd_step(wv[u], step, G));
+                        __stcs(wq + idx, sgd_step(wv[u], step, G[u]));
                     }
                 }
-                if (TB) __stcs(reinterpret_cast<uint16_t *>(n.ebar) + d.q0 + idx, float_to_trace16(ebar, TB));
-                else __stcs(reinterpret_cast<float *>(n.ebar) + d.q0 + idx, ebar);
-                if (ALIF) store_trace(n.epsa, d.q0 + idx, epsa, TB);
-                if (n.record_grad) gq[idx] = grad_add(gq[idx], n.inv_B, G);
+                if (TB) __stcs(reinterpret_cast<uint16_t *>(n.ebar) + d.q0 + idx, float_to_trace16(eb[u], TB));
+                else __stcs(reinterpret_cast<float *>(n.ebar) + d.q0 + idx, eb[u]);
+                if (ALIF) store_trace(n.epsa, d.q0 + idx, ep[u], TB);
+                if (n.record_grad) gq[idx] = grad_add(gq[idx], n.inv_B, G[u]);
             }
         }
         __syncwarp();
