@@ -420,7 +420,7 @@ __host__ __device__ constexpr size_t deliver_stage_bytes(bool state) {
 // last arrival is added on the fly (read-only).  Arrivals are summed in
 // exact int64 fixed point.
 template <bool ALIF, bool STATE>
-__global__ void __launch_bounds__(256, STATE ? 2 : 4) deliver_kernel(Net n, int i) {
+__global__ void __launch_bounds__(256, STATE ? 2 : 4) deliver_kernel(Net n, int i, int part_shift) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ uint64_t bars[8][kDStages];
     __shared__ StageDesc desc[8][kDStages];
@@ -463,11 +463,10 @@ __global__ void __launch_bounds__(256, STATE ? 2 : 4) deliver_kernel(Net n, int 
     const int gw = blockIdx.x * (blockDim.x >> 5) + warp;
     const int nw = gridDim.x * (blockDim.x >> 5);
     // producer cursor (warp-uniform)
-    // work items: (spiking row, one of kDParts equal parts of its synapses),
-    // dealt round-robin to the warps; a step has about as many spiking rows
-    // as there are warps, and whole rows would leave most warps idle while
-    // a few finish a second row
-    constexpr int kDParts = 4;
+    // work items: (spiking row, one of 2^part_shift equal parts of its
+    // synapses), dealt round-robin to the warps; a step has about as many
+    // spiking rows as there are warps, and whole rows would leave most warps
+    // idle while a few finish a second row (host rule: launch_deliver)
     int prow = gw;
     long long pq = 0, pre = 0;
     int psrc = -1, pfirst = 0;
@@ -475,12 +474,12 @@ __global__ void __launch_bounds__(256, STATE ? 2 : 4) deliver_kernel(Net n, int 
     unsigned vmask = 0;
     auto next_item = [&]() -> bool {
         while (pq >= pre) {
-            if (prow >= bs.total * kDParts) return false;
-            const int row = prow / kDParts, part = prow % kDParts;
+            if (prow >= bs.total << part_shift) return false;
+            const int row = prow >> part_shift, part = prow & ((1 << part_shift) - 1);
             psrc = bucket_entry(n, ids, bs, row);
             const long long rb = n.row_ptr[psrc], len = n.row_ptr[psrc + 1] - rb;
-            pq = rb + len * part / kDParts;
-            pre = rb + len * (part + 1) / kDParts;
+            pq = rb + ((len * part) >> part_shift);
+            pre = rb + ((len * (part + 1)) >> part_shift);
             prow += nw;
             pfirst = 1;
             if (STATE && pre > pq && lane >= 1 && lane <= n.D)
@@ -769,13 +768,19 @@ void launch_pred_apply(const Net &n, int i, cudaStream_t st) {
 
 void launch_deliver(const Net &n, int i, int grid_x, cudaStream_t st) {
     const dim3 grid(grid_x, n.B);
+    // four parts per row, more on long rows (at least 512 records each): quarter
+    // rows of 10,000 synapses kept 2.1 blocks busy per SM on average but three on
+    // some, and those set the time (scaling network 84.8 -> 72 ms per call; at 1000
+    // synapses per row 4 parts measured best)
+    int ps = 2;
+    while (((long long)n.segs * kSeg >> (ps + 1)) >= 512 && ps < 10) ++ps;
     if (n.has_state && !n.dense) {
         const size_t sm = deliver_stage_bytes(true) * 8 * kDStages;
-        if (n.alif) launch_pdl(deliver_kernel<true, true>, grid, dim3(256), sm, st, n, i);
-        else launch_pdl(deliver_kernel<false, true>, grid, dim3(256), sm, st, n, i);
+        if (n.alif) launch_pdl(deliver_kernel<true, true>, grid, dim3(256), sm, st, n, i, ps);
+        else launch_pdl(deliver_kernel<false, true>, grid, dim3(256), sm, st, n, i, ps);
     } else {
         const size_t sm = deliver_stage_bytes(false) * 8 * kDStages;
-        launch_pdl(deliver_kernel<false, false>, grid, dim3(256), sm, st, n, i);
+        launch_pdl(deliver_kernel<false, false>, grid, dim3(256), sm, st, n, i, ps);
     }
 }
 
