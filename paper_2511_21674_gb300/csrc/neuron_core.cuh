@@ -33,14 +33,14 @@ __device__ __forceinline__ int drive_count(const Net &n, int b, int j, long long
 // spike-threshold-adaptation, the surrogate).  forced_z >= 0 gives the spike.
 // VAR: the e-prop+ variants (fixed reset, ignore-and-fire, exponential
 // surrogate, rate regularisation) are compiled in; the plain method's
-// instance carries none of their code.
-template <bool VAR>
+// instance carries none of their code.  DRIVE: the external drive is.
+template <bool VAR, bool DRIVE = true>
 __device__ __forceinline__ void neuron_core(const Net &n, int j, long long t_abs, int cnt, long long acc_q,
                                             int forced_z, NeuronRegs &s, float &psi, int &z) {
     // exact fixed-point input split into an FP32 pair
     float u_hi, u_lo;
     fixed_to_pair(acc_q, u_hi, u_lo);
-    if (n.n_thr > 0) {
+    if (DRIVE && n.n_thr > 0) {
         const float dv = n.drive_weight * (float)cnt;
         const float de = fmaf(n.drive_weight, (float)cnt, -dv);
         float e;
