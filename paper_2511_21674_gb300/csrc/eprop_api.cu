@@ -622,14 +622,18 @@ extern "C" eprop_status eprop_set_inputs_targets(eprop_net *net, const int64_t *
     if (!is_device) {
         if (in_step_ptr[0] != 0 || in_step_ptr[B * T] != n_in_ids)
             return fail(net, EPROP_EINVAL, "in_step_ptr must run from 0 to n_in_ids");
-        long long mx = 0;
+        // extremes first, one check after: loops without exits vectorise (2.6e5
+        // ids per batch of 64 samples)
+        long long mx = 0, mn = 0;
         for (long long q = 0; q < B * T; ++q) {
             const long long d = in_step_ptr[q + 1] - in_step_ptr[q];
-            if (d < 0) return fail(net, EPROP_EINVAL, "in_step_ptr must be non-decreasing");
-            if (d > mx) mx = d;
+            mx = std::max(mx, d);
+            mn = std::min(mn, d);
         }
-        for (long long q = 0; q < n_in_ids; ++q)
-            if (in_ids[q] < 0 || in_ids[q] >= c.n_in) return fail(net, EPROP_EINVAL, "input id out of [0, n_in)");
+        if (mn < 0) return fail(net, EPROP_EINVAL, "in_step_ptr must be non-decreasing");
+        unsigned top = 0;                    // negative ids are large as unsigned
+        for (long long q = 0; q < n_in_ids; ++q) top = std::max(top, (unsigned)in_ids[q]);
+        if (n_in_ids > 0 && (long long)top >= c.n_in) return fail(net, EPROP_EINVAL, "input id out of [0, n_in)");
         if (lengths)
             for (long long b = 0; b < B; ++b)
                 if (lengths[b] < 1 || lengths[b] > T) return fail(net, EPROP_EINVAL, "lengths must be in [1, T]");
