@@ -256,10 +256,10 @@ __global__ void __launch_bounds__(kLsThreads) learning_signal_kernel(const float
 // the million-neuron workload's window).  One CTA per SM walks tiles of 128
 // neurons; the window's E is split into TF32 hi + lo once and stays in
 // shared memory.  Roles run concurrently, joined by mbarriers:
-//   warps 4-7  producers: each feedback chunk (128 rows x 32) is loaded
-//              (registers one chunk ahead), split and stored into one of two
-//              operand stages; arrive on full[stage];
-//   warp 8     one thread issues the chunk's products into one of two
+//   warps 4-11 producers: each feedback chunk (128 rows x 32) is loaded
+//              (registers, kLsAhead chunks ahead), split and stored into one of
+//              two operand stages; arrive on full[stage];
+//   warp 12    one thread issues the chunk's products into one of two
 //              accumulator pairs in TMEM and commits to empty[stage], and at
 //              a tile's end to acc_full[pair];
 //   warps 0-3  epilogue: read a finished accumulator pair (TMEM lanes 32 w ..
@@ -270,7 +270,10 @@ __global__ void __launch_bounds__(kLsThreads) learning_signal_kernel(const float
 // learning_signal_kernel.  Every wait is bounded; a wait that gives up
 // raises a CTA-wide abort flag that every role checks.
 constexpr int kLsPKC = 4;                          // K-chunks kept resident (K <= 128)
-constexpr int kLsWThreads = 288;                   // 9 warps
+constexpr int kLsProd = 8;                         // producer warps
+constexpr int kLsAhead = 3;                        // chunks each producer has in flight in registers
+constexpr int kLsRows = kLsM / kLsProd;            // rows of a chunk per producer
+constexpr int kLsWThreads = (4 + kLsProd + 1) * 32;
 constexpr int kLsWStages = 2;
 constexpr size_t kLsWSmem = 1024 + (size_t)kLsPKC * 2 * kLsEreg + (size_t)kLsWStages * 2 * kLsAreg;
 static_assert(kLsWSmem <= 200 * 1024, "warp-specialised learning-signal buffers exceed the request");
@@ -309,7 +312,7 @@ __global__ void __launch_bounds__(kLsWThreads, 1)
     if (warp == 0) tmem_alloc(&tmem_slot, ncols);
     if (tid == 0) {
         for (int q2 = 0; q2 < kLsWStages; ++q2) {
-            mbar_init(&full[q2], 4);                  // one arrival per producer warp
+            mbar_init(&full[q2], kLsProd);            // one arrival per producer warp
             mbar_init(&empty[q2], 1);                 // the products' commit
         }
         for (int q2 = 0; q2 < 2; ++q2) {
@@ -346,36 +349,47 @@ __global__ void __launch_bounds__(kLsWThreads, 1)
     long long n_my = 0;                               // tiles of this CTA
     for (int t = blockIdx.x; t < tiles; t += gridDim.x) ++n_my;
     long long last_commit = -1;                       // products: chunks committed
-    if (warp >= 4 && warp < 8) {
-        // ---- producers: 128 threads, thread (pw, lane) owns rows pw + 4 i
+    if (warp >= 4 && warp < 4 + kLsProd) {
+        // ---- producers: thread (pw, lane) owns rows pw + kLsProd i
         const int pw = warp - 4;
-        float pre[kLsM / 4];
-        auto load_chunk = [&](long long c) {
+        float pre[kLsAhead][kLsRows];
+        auto load_chunk = [&](long long c, float (&x)[kLsRows]) {
             const long long tl = c / nkc;
             const int kc = (int)(c % nkc);
             const int j0 = (int)(blockIdx.x + tl * gridDim.x) * kLsM;
             const int k = kc * kLsKC + lane;
             const bool use = tl < n_my && k < K;
 #pragma unroll
-            for (int i = 0; i < kLsM / 4; ++i) {
-                const int j = j0 + pw + 4 * i;
-                pre[i] = (use && j < N) ? __ldg(fb + (long long)j * K + k) : 0.f;
+            for (int i = 0; i < kLsRows; ++i) {
+                const int j = j0 + pw + kLsProd * i;
+                x[i] = (use && j < N) ? __ldg(fb + (long long)j * K + k) : 0.f;
             }
         };
         const long long nch = n_my * nkc;
-        if (nch > 0) load_chunk(0);
-        for (long long c = 0; c < nch; ++c) {
-            const int st = (int)(c % kLsWStages);
-            if (c >= kLsWStages && !wait(&empty[st], (uint32_t)(((c / kLsWStages) - 1) & 1))) break;
-            unsigned char *ah = a_base + (size_t)(2 * st) * kLsAreg, *al = a_base + (size_t)(2 * st + 1) * kLsAreg;
 #pragma unroll
-            for (int i = 0; i < kLsM / 4; ++i) put_split(ah, al, sw128_off(pw + 4 * i, lane), pre[i]);
-            if (c + 1 < nch) load_chunk(c + 1);
-            fence_proxy_async();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cta(&full[st]);
+        for (int d = 0; d < kLsAhead; ++d)
+            if (d < nch) load_chunk(d, pre[d]);
+        bool okc = true;
+        for (long long c0 = 0; c0 < nch && okc; c0 += kLsAhead) {
+#pragma unroll
+            for (int d = 0; d < kLsAhead; ++d) {
+                const long long c = c0 + d;
+                if (c >= nch || !okc) break;
+                const int st = (int)(c % kLsWStages);
+                if (c >= kLsWStages && !wait(&empty[st], (uint32_t)(((c / kLsWStages) - 1) & 1))) {
+                    okc = false;
+                    break;
+                }
+                unsigned char *ah = a_base + (size_t)(2 * st) * kLsAreg, *al = a_base + (size_t)(2 * st + 1) * kLsAreg;
+#pragma unroll
+                for (int i = 0; i < kLsRows; ++i) put_split(ah, al, sw128_off(pw + kLsProd * i, lane), pre[d][i]);
+                if (c + kLsAhead < nch) load_chunk(c + kLsAhead, pre[d]);
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cta(&full[st]);
+            }
         }
-    } else if (warp == 8) {
+    } else if (warp == 4 + kLsProd) {
         // ---- products: the whole warp follows the barriers (it stays
         // converged), lane 0 issues
         const uint32_t idesc = idesc_tf32(kLsM, npad);
@@ -442,7 +456,7 @@ __global__ void __launch_bounds__(kLsWThreads, 1)
     }
     // products in flight when a wait gave up: one more bounded wait on the
     // last commit before the accumulators are released
-    if (warp == 8 && lane == 0 && s_abort && last_commit >= 0) {
+    if (warp == 4 + kLsProd && lane == 0 && s_abort && last_commit >= 0) {
         const int st = (int)(last_commit % kLsWStages);
         for (unsigned it2 = 0; it2 < kWaitLimit; ++it2)
             if (mbar_try_wait(&empty[st], (uint32_t)((last_commit / kLsWStages) & 1))) break;
