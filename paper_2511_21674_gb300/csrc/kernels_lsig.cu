@@ -291,6 +291,10 @@ __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&v)[1
         : "memory");
 }
 
+// VEC: the feedback rows are 16-byte aligned (K a multiple of 4), so a lane
+// loads, splits and stores four consecutive elements at a time (a quarter of
+// the load, address and store instructions, which bound the producers).
+template <bool VEC>
 __global__ void __launch_bounds__(kLsWThreads, 1)
     learning_signal_ws_kernel(const float *__restrict__ fb, const float *__restrict__ E, float *__restrict__ L,
                               int N, int U, int K, unsigned *err) {
@@ -350,19 +354,53 @@ __global__ void __launch_bounds__(kLsWThreads, 1)
     for (int t = blockIdx.x; t < tiles; t += gridDim.x) ++n_my;
     long long last_commit = -1;                       // products: chunks committed
     if (warp >= 4 && warp < 4 + kLsProd) {
-        // ---- producers: thread (pw, lane) owns rows pw + kLsProd i
+        // ---- producers: scalar form, thread (pw, lane) owns element lane of
+        // rows pw + kLsProd i; vector form, elements 4 (lane % 8) .. + 3 of
+        // rows 16 pw + 4 i + lane / 8
         const int pw = warp - 4;
         float pre[kLsAhead][kLsRows];
         auto load_chunk = [&](long long c, float (&x)[kLsRows]) {
             const long long tl = c / nkc;
             const int kc = (int)(c % nkc);
             const int j0 = (int)(blockIdx.x + tl * gridDim.x) * kLsM;
-            const int k = kc * kLsKC + lane;
-            const bool use = tl < n_my && k < K;
+            if (VEC) {
+                const int k = kc * kLsKC + 4 * (lane & 7);
+                const int jr = j0 + kLsRows * pw + (lane >> 3);
+                const float *src = fb + (long long)jr * K + k;
+                const bool use = tl < n_my && k < K;
 #pragma unroll
-            for (int i = 0; i < kLsRows; ++i) {
-                const int j = j0 + pw + kLsProd * i;
-                x[i] = (use && j < N) ? __ldg(fb + (long long)j * K + k) : 0.f;
+                for (int i = 0; i < kLsRows / 4; ++i) {
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (use && jr + 4 * i < N) v = __ldg(reinterpret_cast<const float4 *>(src + 4 * i * K));
+                    x[4 * i] = v.x; x[4 * i + 1] = v.y; x[4 * i + 2] = v.z; x[4 * i + 3] = v.w;
+                }
+            } else {
+                const int k = kc * kLsKC + lane;
+                const bool use = tl < n_my && k < K;
+#pragma unroll
+                for (int i = 0; i < kLsRows; ++i) {
+                    const int j = j0 + pw + kLsProd * i;
+                    x[i] = (use && j < N) ? __ldg(fb + (long long)j * K + k) : 0.f;
+                }
+            }
+        };
+        auto store_chunk = [&](unsigned char *ah, unsigned char *al, const float (&x)[kLsRows]) {
+            if (VEC) {
+#pragma unroll
+                for (int i = 0; i < kLsRows / 4; ++i) {
+                    uint32_t h[4], l[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        h[e] = tf32_rna(x[4 * i + e]);
+                        l[e] = tf32_rna(x[4 * i + e] - __uint_as_float(h[e]));
+                    }
+                    const uint32_t off = sw128_off(kLsRows * pw + 4 * i + (lane >> 3), 4 * (lane & 7));
+                    *reinterpret_cast<uint4 *>(ah + off) = make_uint4(h[0], h[1], h[2], h[3]);
+                    *reinterpret_cast<uint4 *>(al + off) = make_uint4(l[0], l[1], l[2], l[3]);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < kLsRows; ++i) put_split(ah, al, sw128_off(pw + kLsProd * i, lane), x[i]);
             }
         };
         const long long nch = n_my * nkc;
@@ -381,8 +419,7 @@ __global__ void __launch_bounds__(kLsWThreads, 1)
                     break;
                 }
                 unsigned char *ah = a_base + (size_t)(2 * st) * kLsAreg, *al = a_base + (size_t)(2 * st + 1) * kLsAreg;
-#pragma unroll
-                for (int i = 0; i < kLsRows; ++i) put_split(ah, al, sw128_off(pw + kLsProd * i, lane), pre[d][i]);
+                store_chunk(ah, al, pre[d]);
                 if (c + kLsAhead < nch) load_chunk(c + kLsAhead, pre[d]);
                 fence_proxy_async();
                 __syncwarp();
@@ -442,10 +479,14 @@ __global__ void __launch_bounds__(kLsWThreads, 1)
                 tmem_ld16_nowait(ta0 + half + (uint32_t)(16 * g), w);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                 if (j < N) {
+                    float *dst = L + (long long)(16 * g) * N + j;
+                    if (16 * g + 16 <= U) {
 #pragma unroll
-                    for (int c2 = 0; c2 < 16; ++c2) {
-                        const int u = 16 * g + c2;
-                        if (u < U) L[(long long)u * N + j] = __uint_as_float(v[c2]) + __uint_as_float(w[c2]);
+                        for (int c2 = 0; c2 < 16; ++c2, dst += N) *dst = __uint_as_float(v[c2]) + __uint_as_float(w[c2]);
+                    } else {
+#pragma unroll
+                        for (int c2 = 0; c2 < 16; ++c2, dst += N)
+                            if (16 * g + c2 < U) *dst = __uint_as_float(v[c2]) + __uint_as_float(w[c2]);
                     }
                 }
             }
@@ -471,7 +512,8 @@ __global__ void __launch_bounds__(kLsWThreads, 1)
 
 void prepare_learning_signal_attributes() {
     cudaFuncSetAttribute(learning_signal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLsSmem);
-    cudaFuncSetAttribute(learning_signal_ws_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLsWSmem);
+    cudaFuncSetAttribute(learning_signal_ws_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLsWSmem);
+    cudaFuncSetAttribute(learning_signal_ws_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLsWSmem);
 }
 
 void launch_learning_signals(const float *fb, const float *E, float *L, int N, int U, int K, int B,
@@ -482,7 +524,11 @@ void launch_learning_signals(const float *fb, const float *E, float *L, int N, i
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const int tiles = (N + kLsM - 1) / kLsM;
-        learning_signal_ws_kernel<<<tiles < sms ? tiles : sms, kLsWThreads, kLsWSmem, st>>>(fb, E, L, N, U, K, err);
+        const int grid = tiles < sms ? tiles : sms;
+        if (K % 4 == 0 && (reinterpret_cast<uintptr_t>(fb) & 15) == 0)
+            learning_signal_ws_kernel<true><<<grid, kLsWThreads, kLsWSmem, st>>>(fb, E, L, N, U, K, err);
+        else
+            learning_signal_ws_kernel<false><<<grid, kLsWThreads, kLsWSmem, st>>>(fb, E, L, N, U, K, err);
         return;
     }
     const dim3 grid((unsigned)((N + kLsM - 1) / kLsM), (unsigned)B);
