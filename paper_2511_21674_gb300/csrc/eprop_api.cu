@@ -523,7 +523,7 @@ extern "C" eprop_status eprop_create_network(const eprop_config *cfg, const epro
         FA(v_lo, float, B * N);
         FA(a_lo, float, B * N);
         FA(ref, int, B * N);
-        FA(z_prev, uint8_t, B * N);
+        FA(z_prev, uint8_t, B * N + 4);
         FA(ring, long long, B * (c.max_delay + 1) * N);
         FA(anchor_t, int, B * S);
         FA(anchor_z, float, B * S);
@@ -720,22 +720,30 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
     const long long B = c.batch, N = c.n_rec, K = c.n_out, S = n.n_src;
     const int U = n.U;
     if (!c.continuous) {
-        cudaMemsetAsync(n.v, 0, B * N * 4, st);
-        cudaMemsetAsync(n.a, 0, B * N * 4, st);
-        cudaMemsetAsync(n.v_lo, 0, B * N * 4, st);
-        cudaMemsetAsync(n.a_lo, 0, B * N * 4, st);
-        cudaMemsetAsync(n.ref, 0, B * N * 4, st);
-        cudaMemsetAsync(n.z_prev, 0, B * N, st);
-        cudaMemsetAsync(n.ring, 0, B * (n.D + 1) * N * 8, st);
-        cudaMemsetAsync(n.bits, 0, B * S * n.RW * 4, st);
-        cudaMemsetAsync(n.list_cnt, 0, B * n.RS * eprop::kBkt * 4, st);
-        cudaMemsetAsync(n.y, 0, B * K * 4, st);
-        cudaMemsetAsync(n.y_acc, 0, B * K * 8, st);
-        cudaMemsetAsync(n.zk, 0, 2 * B * N * 4, st);
-        cudaMemsetAsync(n.psi_hist, 0, B * (U + 1) * N * 4, st);
-        cudaMemsetAsync(n.anchor_z, 0, B * S * 4, st);
-        if (n.rate) cudaMemsetAsync(n.rate, 0, B * N * 4, st);
-        eprop::launch_fill_int(n.anchor_t, B * S, eprop::kNoSpike, st);
+        eprop::ResetList rl;
+        rl.add(n.v, B * N);
+        rl.add(n.v_lo, B * N);
+        if (n.alif) {
+            rl.add(n.a, B * N);
+            rl.add(n.a_lo, B * N);
+        }
+        rl.add(n.ref, B * N);
+        rl.add(n.z_prev, (B * N + 3) / 4);               // (its allocation is padded)
+        rl.add(n.ring, B * (n.D + 1) * N * 2);
+        rl.add(n.bits, B * S * n.RW);
+        rl.add(n.list_cnt, B * n.RS * eprop::kBkt);
+        rl.add(n.y, B * K);
+        rl.add(n.y_acc, B * K * 2);
+        rl.add(n.zk, 2 * B * N);
+        rl.add(n.psi_hist, N, 0, B, (long long)(U + 1) * N);     // slot 0; the steps write the others
+        rl.add(n.anchor_z, B * S);
+        rl.add(n.anchor_t, B * S, eprop::kNoSpike);
+        if (n.rate) rl.add(n.rate, B * N);
+        if (n.pred_mode) {
+            rl.add(n.pop_rate, B * eprop::kPopGroups);
+            rl.add(n.pop_cnt, B * eprop::kPopGroups);
+        }
+        eprop::launch_reset(rl, net->sm_count, st);
         if (n.has_state) {
             const size_t tb = n.trace_bf16 ? 2 : 4;
             const long long nt = n.band ? n.nnz_b : n.nnz;
@@ -744,12 +752,8 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
         }
     }
     if (n.record_raster) cudaMemsetAsync(n.rec_raster, 0, B * ((T + 31) / 32) * N * 4, st);
-    if (n.pred_mode && !c.continuous) {
-        cudaMemsetAsync(n.pop_rate, 0, B * eprop::kPopGroups * 4, st);
-        cudaMemsetAsync(n.pop_cnt, 0, B * eprop::kPopGroups * 4, st);
-    }
     long long L = 0, LT = 0, nwin = 0;
-    if (!c.continuous) L += 1;                       // anchor fill
+    if (!c.continuous) L += 1;                       // reset
     eprop::launch_begin_call(n, c.continuous, st);
     L += 1;
     // the delivery and trace kernels hold two 256-thread blocks per SM (launch

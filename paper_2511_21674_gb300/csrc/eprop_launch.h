@@ -34,6 +34,21 @@ void launch_rollover(const Net &n, int i_end, cudaStream_t st);
 void launch_flush(const Net &n, int i_end, float *w_dst, float *g_dst, long long q_begin, long long q_end,
                   int write_back, int sm_count, cudaStream_t st);
 void launch_fill_int(int *p, long long count, int value, cudaStream_t st);
+// ranges of 4-byte words set to a value in one launch: `rows` runs of `words`,
+// `stride` words apart
+struct ResetRange {
+    int *p;
+    long long words, rows, stride;
+    int value;
+};
+struct ResetList {
+    int n = 0;
+    ResetRange r[20];
+    void add(void *p, long long words, int value = 0, long long rows = 1, long long stride = 0) {
+        if (words > 0) r[n++] = ResetRange{static_cast<int *>(p), words, rows, stride, value};
+    }
+};
+void launch_reset(const ResetList &l, int sm_count, cudaStream_t st);
 void launch_unpack_raster(const Net &n, unsigned char *dst, cudaStream_t st);
 void launch_adam(const Net &n, int sm_count, cudaStream_t st);
 int persistent_blocks(int sm_count);
