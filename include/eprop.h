@@ -143,15 +143,20 @@ typedef struct eprop_config {
                                  1: capture a call once in a CUDA graph and
                                  replay it for later calls with the same T;
                                  2: as 1, with every step of the call in one
-                                 persistent cooperative kernel (grid barriers
-                                 between the neuron and the delivery phases,
-                                 bounded waits: EPROP_ETIMEOUT); needs one
+                                 launch: a small network (see trace_kernel)
+                                 sample by sample, one block each (it runs so
+                                 in every launch mode, window by window), a
+                                 larger one in a persistent cooperative kernel
+                                 (grid barriers between the neuron and the
+                                 delivery phases, bounded waits:
+                                 EPROP_ETIMEOUT); needs one
                                  update window per call (continuous = 0,
                                  update_interval = 0), n_out <= 256 and no
                                  predictor; results are bit-identical to 0/1 */
     int32_t trace_kernel;     /* synapse-trace kernel: 0 auto (3 when state is
                                  carried, else 2 for batch > 1 or a small network
-                                 (n_rec <= 1024, <= 2^21 synapses), else 1);
+                                 (n_rec <= 1024, <= 2^19 recurrent and 2^21
+                                 synapses in all), else 1);
                                  1 lazy window work queue (batch 1): only
                                  synapses with an arrival are touched, a
                                  skipped window is caught up at the next

@@ -39,7 +39,8 @@ namespace eprop {
 constexpr int kSmpMaxOut = 128;        // readouts: at most 4 readout warps
 constexpr int kSmpMaxRec = 1024;
 constexpr int kSmpMaxIn = 32768;
-constexpr long long kSmpMaxNnz = 1LL << 21;
+constexpr long long kSmpMaxNnz = 1LL << 21;      // all synapses
+constexpr long long kSmpMaxNnzRec = 1LL << 19;   // recurrent synapses
 constexpr int kSmpPart = 128;          // records of a row per delivery item: 4 per lane in flight
 
 struct SampleShape {
@@ -519,11 +520,17 @@ __global__ void __launch_bounds__(BT, 1) sample_steps_kernel(Net n, int i0, int 
     if (lists && tid < kBkt) n.list_cnt[list_index(n, b, (ck.r_base + i1 + 1) % n.RS) + tid] = 0;
 }
 
-// One thread per neuron (at most four), synapses that fit one SM's L1/L2
-// share and whose per-step events one SM adds faster than a step's launches
-// take.
+// One thread per neuron (at most four), row starts in 32 bits, and events that
+// one SM adds faster than a step's launches take.  The last is a matter of the
+// recurrent synapses (a step of a strongly active network touches some percent
+// of them); measured per call, this loop against the per-step kernels, all-to-
+// all networks at 9e2 / 4e3 / 1e4 / 3.4e4 events per step: 100 neurons x 300 steps
+// 0.35 / 3.8 ms, 400 1.2 / 4.1, 700 (4.9e5 synapses) 2.1 / 4.5, 1024 (1.05e6) 5.8 /
+// 4.7.  With 10 % recurrent and 2312 inputs (100 steps): 600 neurons 0.77 / 1.5 (one
+// sample), 850 neurons (2e6 synapses) x 64 samples 1.2 / 2.5.
 bool sample_net_small(const Net &n) {
-    return n.n_rec <= kSmpMaxRec && n.n_in <= kSmpMaxIn && n.n_out <= kSmpMaxOut && n.nnz <= kSmpMaxNnz;
+    return n.n_rec <= kSmpMaxRec && n.n_in <= kSmpMaxIn && n.n_out <= kSmpMaxOut && n.nnz <= kSmpMaxNnz &&
+           n.nnz - n.nnz_in <= kSmpMaxNnzRec;
 }
 bool sample_steps_fit(const Net &n) {
     return sample_net_small(n) && n.pred_mode == 0 && n.d_out == 0 && !n.band && !(n.has_state && !n.dense);

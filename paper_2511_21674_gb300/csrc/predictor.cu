@@ -28,10 +28,9 @@ struct eprop_predictor {
     bf16 *Wh[3] = {nullptr, nullptr, nullptr};
     bf16 *Xh = nullptr, *H1h = nullptr, *H2h = nullptr, *dYh = nullptr, *dA2h = nullptr, *dA1h = nullptr;
     float *A1 = nullptr, *A2 = nullptr, *Y = nullptr;
-    float *gpart = nullptr;          // [kMaxSlices][n_params] weight gradients of row slices
     float *bpart = nullptr;          // [row tiles][2 hidden + n_out] bias gradients of row tiles
     float *lpart = nullptr;          // [row tiles] squared errors
-    int sm_count = 1, max_slices = 1;
+    int sm_count = 1;
     float *xin = nullptr, *ein = nullptr, *yout = nullptr, *loss = nullptr;
     float *stage = nullptr;          // FP32 widening of BF16 buffers for eprop_predictor_read
     float *in_scale = nullptr;       // [n_in] input scale (part of the model; default 1)
@@ -287,82 +286,76 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_kernel(Mlp a) {
 }
 
 // Weight gradients dW[m][n] = sum_r A[r][m] D[r][n] of the three layers in one
-// launch: block = (64 x 64 tile of a layer, slice of the rows); the slices'
-// sums are added in order by the Adam kernel.  One block per tile over all
-// 4096 rows left 32 blocks busy for 678 us.
-constexpr int kDwThreads = 128, kDwTile = 64, kDwStages = 4, kDwLd = kDwTile + 8;
+// launch, one block per 32 x 32 tile over all rows.  The rows are not split: one
+// accumulator per element, 16 rows per step in row order, keeps the sums' bits
+// (Adam divides small gradients by their own size, so a changed last bit of a
+// gradient near zero would move its weight), and with eight chunks of 64 rows
+// in flight the walk is bound by L2, not by its length.  64 x 32 tiles with
+// element-wise staging took 678 us per layer at 4096 rows; this launch 21 us
+// for all three.
+constexpr int kDwThreads = 128, kDwTile = 32, kDwRows = 64, kDwStages = 8, kDwLd = kDwTile + 8;
 struct Dw {
-    int rows, slice, tiles[3];
+    int rows, tiles[3];
     const bf16 *A[3], *D[3];
     int ldA[3], ldD[3], M[3], N[3];
-    long long off[3], n_params;
-    float *part;
+    float *out[3];
 };
 
 __global__ void __launch_bounds__(kDwThreads) dw_kernel(Dw a) {
     extern __shared__ __align__(16) unsigned char pred_sm[];
     bf16 *ring = reinterpret_cast<bf16 *>(pred_sm);
-    constexpr int kStage = 2 * kDwTile * kDwLd;
+    constexpr int kStage = 2 * kDwRows * kDwLd;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     int l = 0, tile = blockIdx.x;
     while (l < 2 && tile >= a.tiles[l]) tile -= a.tiles[l++];
     const int M = a.M[l], N = a.N[l], nt = (N + kDwTile - 1) / kDwTile;
     const int m0 = tile / nt * kDwTile, n0 = tile % nt * kDwTile;
-    const int rb = blockIdx.y * a.slice, re = min(a.rows, rb + a.slice);
-    const int chunks = (re - rb + kDwTile - 1) / kDwTile;
+    const int chunks = (a.rows + kDwRows - 1) / kDwRows;
     auto load = [&](int c) {
         if (c < chunks) {
             bf16 *st = ring + (c % kDwStages) * kStage;
-            for (int q = tid; q < 2 * kDwTile * 8; q += kDwThreads) {
-                const int which = q / (kDwTile * 8), k = (q >> 3) % kDwTile, cc = (q & 7) * 8;
+#pragma unroll
+            for (int q = tid; q < 2 * kDwRows * (kDwTile / 8); q += kDwThreads) {
+                const int which = q / (kDwRows * (kDwTile / 8)), k = (q / (kDwTile / 8)) % kDwRows;
+                const int cc = (q % (kDwTile / 8)) * 8;
                 const bf16 *src = which ? a.D[l] : a.A[l];
-                const int ld = which ? a.ldD[l] : a.ldA[l], c0 = (which ? n0 : m0) + cc, r = rb + c * kDwTile + k;
-                const bool in = r < re && c0 < ld;
-                cp16(st + which * kDwTile * kDwLd + k * kDwLd + cc, in ? src + (size_t)r * ld + c0 : src, in);
+                const int ld = which ? a.ldD[l] : a.ldA[l], c0 = (which ? n0 : m0) + cc, r = c * kDwRows + k;
+                const bool in = r < a.rows && c0 < ld;
+                cp16(st + which * kDwRows * kDwLd + k * kDwLd + cc, in ? src + (size_t)r * ld + c0 : src, in);
             }
         }
         cp_commit();
     };
     for (int c = 0; c < kDwStages - 1; ++c) load(c);
-    float acc[2][4][4];
+    float acc[2][4];
 #pragma unroll
-    for (int m = 0; m < 2; ++m)
+    for (int j = 0; j < 2; ++j)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[m][j][e] = 0.f;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32, mt = lane >> 3, lr = lane & 7;
+        for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+    const int wm = (warp >> 1) * 16, wn = (warp & 1) * 16, mt = lane >> 3, lr = lane & 7;
     for (int c = 0; c < chunks; ++c) {
         cp_wait<kDwStages - 2>();
         __syncthreads();
         load(c + kDwStages - 1);
-        const bf16 *As = ring + (c % kDwStages) * kStage, *Ds = As + kDwTile * kDwLd;
+        const bf16 *As = ring + (c % kDwStages) * kStage, *Ds = As + kDwRows * kDwLd;
 #pragma unroll
-        for (int ks = 0; ks < kDwTile / 16; ++ks) {
-            uint32_t af[2][4], bfr[2][4];
-#pragma unroll
-            for (int m = 0; m < 2; ++m)
-                ldm4t(af[m], As + (ks * 16 + (mt >> 1) * 8 + lr) * kDwLd + wm + m * 16 + (mt & 1) * 8);
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-                ldm4t(bfr[h], Ds + (ks * 16 + (mt & 1) * 8 + lr) * kDwLd + wn + h * 16 + (mt >> 1) * 8);
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                for (int m = 0; m < 2; ++m) mma_bf16(acc[m][j], af[m], bfr[j >> 1][(j & 1) * 2], bfr[j >> 1][(j & 1) * 2 + 1]);
+        for (int ks = 0; ks < kDwRows / 16; ++ks) {
+            uint32_t af[4], bfr[4];
+            ldm4t(af, As + (ks * 16 + (mt >> 1) * 8 + lr) * kDwLd + wm + (mt & 1) * 8);
+            ldm4t(bfr, Ds + (ks * 16 + (mt & 1) * 8 + lr) * kDwLd + wn + (mt >> 1) * 8);
+            mma_bf16(acc[0], af, bfr[0], bfr[1]);
+            mma_bf16(acc[1], af, bfr[2], bfr[3]);
         }
     }
     cp_wait<0>();
-    float *out = a.part + (size_t)blockIdx.y * a.n_params + a.off[l];
+    float *out = a.out[l];
 #pragma unroll
-    for (int m = 0; m < 2; ++m)
+    for (int j = 0; j < 2; ++j)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int mm = m0 + wm + m * 16 + g + (e >= 2 ? 8 : 0), nn = n0 + wn + j * 8 + 2 * t + (e & 1);
-                if (mm < M && nn < N) out[(size_t)mm * N + nn] = acc[m][j][e];
-            }
+        for (int e = 0; e < 4; ++e) {
+            const int mm = m0 + wm + g + (e >= 2 ? 8 : 0), nn = n0 + wn + j * 8 + 2 * t + (e & 1);
+            if (mm < M && nn < N) out[(size_t)mm * N + nn] = acc[j][e];
+        }
 }
 
 // layout of the packed parameters: layer l holds W [I_l][O_l] then b [O_l]
@@ -391,11 +384,10 @@ __global__ void refresh_kernel(Layout L, const float *w, long long n) {
     }
 }
 
-// Adam (Eq. adam1, Eq. adam2, Eq. adam) on the FP32 masters: sums the
-// gradient's parts in order (weights: row slices; biases: row tiles), steps,
-// and refreshes the BF16 weights; block 0 also sums the loss.
-__global__ void adam_kernel(Layout L, float *w, float *grad, float *m, float *v, long long n, const float *gpart,
-                            int slices, const float *bpart, const float *lpart, int tiles, float half_inv,
+// Adam (Eq. adam1, Eq. adam2, Eq. adam) on the FP32 masters: sums the bias
+// gradients of the row tiles in order, steps, and refreshes the BF16 weights;
+// block 0 also sums the loss.
+__global__ void adam_kernel(Layout L, float *w, float *grad, float *m, float *v, long long n, const float *bpart, const float *lpart, int tiles, float half_inv,
                             float *loss, float lr, float c1, float c2) {
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
          q += (long long)gridDim.x * blockDim.x) {
@@ -403,17 +395,17 @@ __global__ void adam_kernel(Layout L, float *w, float *grad, float *m, float *v,
         long long i;
         bool bias;
         locate(L, q, l, i, bias);
-        float gq = 0.f;
+        float gq;
         if (bias) {
+            gq = 0.f;
             const long long nb = L.O[0] + L.O[1] + L.O[2];
             const float *bp = bpart + (l == 0 ? 0 : l == 1 ? L.O[0] : L.O[0] + L.O[1]) + i;
 #pragma unroll 8
             for (int s = 0; s < tiles; ++s) gq += bp[s * nb];
+            grad[q] = gq;
         } else {
-#pragma unroll 8
-            for (int s = 0; s < slices; ++s) gq += gpart[s * n + q];
+            gq = grad[q];
         }
-        grad[q] = gq;
         const float mq = 0.9f * m[q] + 0.1f * gq;
         const float vq = 0.999f * v[q] + 0.001f * gq * gq;
         m[q] = mq;
@@ -440,7 +432,7 @@ __global__ void bf16_to_float_kernel(const bf16 *src, int ld, int cols, float *d
 // ------------------------------------------------------------------ host
 
 constexpr int kMlpSmemMax = 220 * 1024;
-constexpr int kDwSmem = kDwStages * 2 * kDwTile * kDwLd * (int)sizeof(bf16);
+constexpr int kDwSmem = kDwStages * 2 * kDwRows * kDwLd * (int)sizeof(bf16);
 
 static unsigned blocks_for(long long n) {
     long long b = (n + 255) / 256;
@@ -526,8 +518,6 @@ extern "C" eprop_status eprop_predictor_create(int32_t n_in, int32_t hidden, int
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, dev);
-    // row slices of the weight gradients: at most 16, and at most 16 MB of parts
-    p->max_slices = (int)std::max(1LL, std::min(16LL, (4LL << 20) / o));
     const long long tiles = (R + 15) / 16;
     if (e == cudaSuccess) e = palloc(p, &p->params, o);
     if (e == cudaSuccess) e = palloc(p, &p->grads, o);
@@ -541,7 +531,6 @@ extern "C" eprop_status eprop_predictor_create(int32_t n_in, int32_t hidden, int
     if (e == cudaSuccess) e = palloc(p, &p->dYh, R * p->ldK);
     if (e == cudaSuccess) e = palloc(p, &p->dA2h, R * p->ldH);
     if (e == cudaSuccess) e = palloc(p, &p->dA1h, R * p->ldH);
-    if (e == cudaSuccess) e = palloc(p, &p->gpart, p->max_slices * o);
     if (e == cudaSuccess) e = palloc(p, &p->bpart, tiles * (2 * H + n_out));
     if (e == cudaSuccess) e = palloc(p, &p->lpart, tiles);
     if (e == cudaSuccess) e = palloc(p, &p->A1, R * H);
@@ -704,29 +693,23 @@ extern "C" eprop_status eprop_predictor_train_step(eprop_predictor *p, const flo
     const int tiles = issue_mlp(p, xd, ed, rows, p->st);
     Dw d{};
     d.rows = rows;
-    // slices of at least 128 rows (two chunks in flight per block)
-    int slices = std::min(p->max_slices, (rows + 127) / 128);
-    d.slice = ((rows + slices - 1) / slices + 15) & ~15;
-    slices = (rows + d.slice - 1) / d.slice;
     const bf16 *A[3] = {p->Xh, p->H1h, p->H2h}, *D[3] = {p->dA1h, p->dA2h, p->dYh};
     const int ldA[3] = {p->ldX, p->ldH, p->ldH}, ldD[3] = {p->ldH, p->ldH, p->ldK};
     const int M[3] = {I, H, H}, N[3] = {H, H, K};
     int blocks = 0;
     for (int l = 0; l < 3; ++l) {
         d.A[l] = A[l]; d.D[l] = D[l]; d.ldA[l] = ldA[l]; d.ldD[l] = ldD[l]; d.M[l] = M[l]; d.N[l] = N[l];
-        d.off[l] = p->off_W[l];
+        d.out[l] = p->grads + p->off_W[l];
         d.tiles[l] = ((M[l] + kDwTile - 1) / kDwTile) * ((N[l] + kDwTile - 1) / kDwTile);
         blocks += d.tiles[l];
     }
-    d.n_params = p->n_params;
-    d.part = p->gpart;
-    dw_kernel<<<dim3(blocks, slices), kDwThreads, kDwSmem, p->st>>>(d);
+    dw_kernel<<<blocks, kDwThreads, kDwSmem, p->st>>>(d);
     // Adam step
     p->adam_t += 1;
     const float c1 = (float)(1.0 - std::pow(0.9, (double)p->adam_t));
     const float c2 = (float)(1.0 - std::pow(0.999, (double)p->adam_t));
     adam_kernel<<<blocks_for(p->n_params), 256, 0, p->st>>>(layout_of(p), p->params, p->grads, p->m, p->v, p->n_params,
-                                                             p->gpart, slices, p->bpart, p->lpart, tiles,
+                                                             p->bpart, p->lpart, tiles,
                                                              0.5f / (float)rows, p->loss, lr, c1, c2);
     PCK(p, cudaGetLastError());
     if (loss_out) {
