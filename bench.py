@@ -320,10 +320,10 @@ def cpu_baseline(args, steps=1):
 
 def batched_form_timing(calls=10, warmup=3):
     """Form (2) on the event-classification workload (batch 64, lengths
-    250-350, 200 ALIF, 2312 inputs): ms per simulate call with every kernel
-    launched eagerly (launch_mode 0), as a graph of per-step launches (1) and
-    with the step loop in one persistent cooperative kernel (2); CUDA events
-    on the network's stream, inputs resident."""
+    250-350, 200 ALIF, 2312 inputs): ms per simulate call launched eagerly
+    (launch_mode 0), as a captured graph (1) and with every step of the call in
+    one launch (2; a network of this size runs so in every mode); CUDA events on
+    the network's stream, inputs resident."""
     import torch
     import paper_2511_21674_gb300 as ep
     from workloads import configs as C

@@ -855,7 +855,7 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
             L += 4;
             if (c.profile) cudaEventRecordWithFlags(net->ev[2 * nwin], st, cudaEventRecordExternal);
             if (net->trace_mode == 1) {
-                eprop::launch_trace_batched(n, net->sm_count, st);
+                eprop::launch_trace_batched(n, B == 1 && c.trace_kernel == 0, net->sm_count, st);
                 LT += 1;
             } else if (net->trace_mode == 2 && B > 1) {
                 eprop::launch_window_batched(n, i, net->sm_count, st);

@@ -19,7 +19,8 @@
 //   per-step spike lists (ring of RS steps) [B][RS][kBkt][cap] i32 with
 //     counts [B][RS][kBkt]: a source appends to bucket (src >> 8) % kBkt, so
 //     the appends of one step spread over kBkt counters
-//   window tables [B][U][N] float2 (LIF: Q, Pe) or float4 (ALIF: Q, Pe, Pa)
+//   window tables [B][U][N] float2 (LIF: Q, Pe) or float4 (ALIF: Q, Pe, Pa);
+//     without carried state one float (Q)
 //   window coefficients (ring of RC windows) [N][RC] float4 (LIF) or
 //     2 x float4 (ALIF): neuron-major, so a catch-up over consecutive
 //     windows reads contiguous entries

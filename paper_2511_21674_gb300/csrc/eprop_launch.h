@@ -25,7 +25,7 @@ void launch_trace_window(const Net &n, int i_end, int grid_x, cudaStream_t st);
 // state per sample and synapse
 constexpr int kBatchWindowMax = 64;
 void launch_window_batched(const Net &n, int i_end, int sm_count, cudaStream_t st);
-void launch_trace_batched(const Net &n, int sm_count, cudaStream_t st);
+void launch_trace_batched(const Net &n, bool plain, int sm_count, cudaStream_t st);
 void launch_window_pass(const Net &n, int i_end, int grid_x, int grid_idle, cudaStream_t st);
 void launch_pred_input(const Net &n, int i, cudaStream_t st);
 void launch_pred_apply(const Net &n, int i, cudaStream_t st);

@@ -1101,7 +1101,7 @@ float G[kB];
 // steps, 140 rows: 2063 -> 74 us.
 constexpr int kTbThreads = 256;
 constexpr int kTbCap = 32 * kTbThreads;          // spikes listed: at least one round of words
-__global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n) {
+__global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool plain) {
     __shared__ int sp[kTbCap];                   // (sample << 20) | step
     __shared__ int wsum[kTbThreads / 32];
     __shared__ float2 red[kTbThreads];
@@ -1163,6 +1163,10 @@ __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n) {
         // threads per synapse group: the row's synapses, rounded up to warps
         int tc = 32;
         while (tc < len && tc < kTbThreads) tc <<= 1;
+        // plain: the FP32 sum in step order, as the work-queue form rounds it (a
+        // single-sample network that the automatic choice brings here keeps
+        // that form's bits)
+        if (plain) tc = kTbThreads;
         const int slices = kTbThreads / tc, slice = tid / tc, tq = tid - slice * tc;
         for (int qc = 0; qc < len; qc += tc) {
             const int qi = qc + tq;
@@ -1178,6 +1182,10 @@ __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n) {
                         const int v = sp[c];
                         const int a = (v & 0xFFFFF) + d;
                         const float x = a <= T ? __ldg(qj + ((long long)(v >> 20) * U + (a - 1)) * N) : 0.f;
+                        if (plain) {
+                            hi += x;
+                            continue;
+                        }
                         float e;
                         two_sum(hi, x, hi, e);
                         lo += e;
@@ -1898,9 +1906,9 @@ void launch_window_batched(const Net &n, int i_end, int sm_count, cudaStream_t s
 #undef EPROP_WB
 }
 
-void launch_trace_batched(const Net &n, int sm_count, cudaStream_t st) {
+void launch_trace_batched(const Net &n, bool plain, int sm_count, cudaStream_t st) {
     const int blocks = n.n_src < 6 * sm_count ? n.n_src : 6 * sm_count;
-    trace_batched_kernel<<<blocks, kTbThreads, 0, st>>>(n);
+    trace_batched_kernel<<<blocks, kTbThreads, 0, st>>>(n, plain);
 }
 
 void launch_readout_weights(const Net &n, int i_end, cudaStream_t st) {
