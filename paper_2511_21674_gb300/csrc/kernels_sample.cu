@@ -19,10 +19,10 @@
 //            window the softmax is skipped (its result is multiplied by zero).
 // Measured (one GB300, whole calls, per-step launches or the cooperative step
 // loop before -> this loop and the window-end kernels of today): 100 LIF, 1000
-// steps 10.4 -> 1.20 ms (about 0.9 us per step); batch of 64, 200 ALIF, 350
-// steps with 13 input events each 7.7 -> 1.22 ms (2.0 us per step, bound by the
+// steps 10.4 -> 1.21 ms (0.92 us per step); batch of 64, 200 ALIF, 350
+// steps with 13 input events each 8.2 -> 1.10 ms (2.0 us per step, bound by the
 // instructions of the input rows); batch of 32, 100 ALIF, 2200 steps 43.1 ->
-// 2.09 ms (0.65 us per step).  With the inputs one step ahead and the readout
+// 2.04 ms (0.62 us per step).  With the inputs one step ahead and the readout
 // summing the spikes itself: 1.34, 1.24 and 2.63 ms.
 // One barrier of the workers (spike list complete) and one of the block per
 // step.  The ring holds two 32-bit words per entry: an arrival's low word is

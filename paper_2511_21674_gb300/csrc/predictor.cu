@@ -181,7 +181,8 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_kernel(Mlp a) {
     Pos p{0, 0, 0};
     for (int c = 0; p.ph < kPhases; ++c) {
         if (a.stages == 4) cp_wait<2>();
-        else cp_wait<1>();
+        else if (a.stages == 3) cp_wait<1>();
+        else cp_wait<0>();
         __syncthreads();                 // chunk c is there, chunk c - 1 and its tiles are done
         {
             const int q = c + a.stages - 1;
@@ -628,11 +629,12 @@ static int issue_mlp(eprop_predictor *p, const float *x, const float *e, int row
     a.A1 = p->A1; a.A2 = p->A2; a.Y = p->Y; a.bpart = p->bpart; a.lpart = p->lpart;
     a.inv = 1.0f / (float)rows;
     const bool train = e != nullptr;
-    // 32-row tiles once 16-row tiles fill the SMs; four ring stages where they fit
+    // 32-row tiles once 16-row tiles fill the SMs; four ring stages where they
+    // fit (two at n_in = hidden = n_out = 1024 in training)
     a.stages = 4;
     int mt = rows > 16 * p->sm_count ? 2 : 1;
     if (mlp_smem(a, mt, train) > (size_t)kMlpSmemMax) mt = 1;
-    if (mlp_smem(a, mt, train) > (size_t)kMlpSmemMax) a.stages = 3;
+    while (a.stages > 2 && mlp_smem(a, mt, train) > (size_t)kMlpSmemMax) --a.stages;
     const int tiles = (rows + 16 * mt - 1) / (16 * mt);
     const size_t sm = mlp_smem(a, mt, train);
     if (train) {

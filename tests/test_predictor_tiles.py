@@ -13,7 +13,8 @@ from tests.test_predictor_gpu import U23, _bf16_check, _gemm_check
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("R,n_in,H,K", [(1, 1, 16, 1), (17, 75, 33, 11), (2600, 20, 300, 5), (40, 1024, 1024, 70)])
+@pytest.mark.parametrize("R,n_in,H,K", [(1, 1, 16, 1), (17, 75, 33, 11), (2600, 20, 300, 5), (40, 1024, 1024, 70),
+                                         (20, 1024, 1024, 1024)])
 def test_train_step_at_tile_edges(R, n_in, H, K):
     import paper_2511_21674_gb300 as ep
     rng = np.random.default_rng(R)
