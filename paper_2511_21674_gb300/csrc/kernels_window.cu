@@ -21,6 +21,7 @@
 
 #include "eprop_internal.cuh"
 #include "eprop_launch.h"
+#include "spike_entry.h"
 
 namespace eprop {
 
@@ -1102,7 +1103,7 @@ float G[kB];
 constexpr int kTbThreads = 256;
 constexpr int kTbCap = 32 * kTbThreads;          // spikes listed: at least one round of words
 __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool plain) {
-    __shared__ int sp[kTbCap];                   // (sample << 20) | step
+    __shared__ uint32_t sp[kTbCap];              // spike_entry.h
     __shared__ int wsum[kTbThreads / 32];
     __shared__ float2 red[kTbThreads];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1113,16 +1114,19 @@ __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool p
         const long long q0 = n.row_ptr[src];
         const int len = (int)(n.row_ptr[src + 1] - q0);
         if (len == 0) continue;
-        // lists the spikes of words w0.. until the list is full; returns the
-        // next word
+        // lists the spikes of words w0.. until the list is full or its entries'
+        // range is used up; returns the next word
         int ns = 0;
+        long long base = 0;
         auto fill = [&](int w0) -> int {
             ns = 0;
-            while (w0 < nwords) {
+            base = entry_base(w0 / wps, w0 % wps, U);
+            const int w_end = nwords - w0 > kEntrySpan ? w0 + kEntrySpan : nwords;
+            while (w0 < w_end) {
                 const int w = w0 + tid;
                 uint32_t m = 0u;
                 int b = 0, k = 0;
-                if (w < nwords) {
+                if (w < w_end) {
                     b = w / wps;
                     k = w - b * wps;
                     m = n.bits[((long long)b * n.n_src + src) * n.RW + k];
@@ -1148,11 +1152,11 @@ __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool p
                 if (ns + all > kTbCap) break;    // (never in the first round)
                 int pos = ns + before + x - c;
                 while (m) {
-                    sp[pos++] = (b << 20) | (k * 32 + __ffs(m) - 1);
+                    sp[pos++] = entry_pack(base, b, k * 32 + __ffs(m) - 1, U, T);
                     m &= m - 1;
                 }
                 ns += all;
-                w0 += kTbThreads;
+                w0 = min(w0 + kTbThreads, w_end);
             }
             __syncthreads();
             return w0;
@@ -1179,9 +1183,8 @@ __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool p
                 if (td != 0u) {
 #pragma unroll 4
                     for (int c = slice; c < ns; c += slices) {
-                        const int v = sp[c];
-                        const int a = (v & 0xFFFFF) + d;
-                        const float x = a <= T ? __ldg(qj + ((long long)(v >> 20) * U + (a - 1)) * N) : 0.f;
+                        const uint32_t v = sp[c];
+                        const float x = entry_arrives(v, d) ? __ldg(qj + entry_row(base, v, d) * N) : 0.f;
                         if (plain) {
                             hi += x;
                             continue;
