@@ -10,6 +10,7 @@
 
 #include "eprop.h"
 #include "eprop_internal.cuh"
+#include "delivery_split.h"
 #include "eprop_launch.h"
 #include "eprop_predictor.h"
 #include "predictor_internal.h"
@@ -26,6 +27,8 @@ struct eprop_net {
     Net n;
     cudaStream_t st = nullptr;
     int dev = 0, sm_count = 1;
+    int part_shift = 2;                          // delivery (delivery_split.h)
+    const eprop::HubRows *hubs = nullptr;
     std::string err;
     int bad = 0;
     std::vector<DevAlloc> fixed_allocs;   // freed at destroy
@@ -468,6 +471,17 @@ extern "C" eprop_status eprop_create_network(const eprop_config *cfg, const epro
             long long mx = 0;
             for (long long i = 0; i < S; ++i) mx = std::max(mx, hp[i + 1] - hp[i]);
             n.segs = (int)std::max(1LL, (mx + eprop::kSeg - 1) / eprop::kSeg);
+            net->part_shift = eprop::delivery_part_shift(nnz, S);
+            eprop::HubRows hubs{eprop::delivery_hub_length(hp.data(), S, net->part_shift), 0, 0, {}};
+            for (long long i = 0; i < S; ++i)
+                if (hp[i + 1] - hp[i] > hubs.len) hubs.src[hubs.n++] = (int)i;
+            hubs.parts = (int)((mx + eprop::kHubPart - 1) / eprop::kHubPart);
+            if (hubs.n > 0) {
+                cudaError_t he = dalloc(o, &p, sizeof(hubs));
+                if (he == cudaSuccess) he = cudaMemcpy(p, &hubs, sizeof(hubs), cudaMemcpyHostToDevice);
+                if (he != cudaSuccess) { s = cuda_fail(nullptr, he, "hub rows"); goto fail_out; }
+                net->hubs = static_cast<const eprop::HubRows *>(p);
+            }
         }
         uint32_t *td;
         FA(tgt_d, uint32_t, nnz + 16);
@@ -838,7 +852,7 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
             }
         }
         if (n.band) eprop::launch_deliver_band(n, i, deliver_rows, st);
-        else eprop::launch_deliver(n, i, deliver_rows, st);
+        else eprop::launch_deliver(n, i, deliver_rows, net->part_shift, net->hubs, st);
         L += 3;
         }
         if (i % U == 0) {

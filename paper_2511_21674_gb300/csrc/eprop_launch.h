@@ -12,7 +12,9 @@ struct GridBar;
 // neuron updates and input spikes of call step i
 void launch_neuron(const Net &n, int i, int max_events_per_step, cudaStream_t st);
 void launch_readout(const Net &n, int i, int sm_count, cudaStream_t st);
-void launch_deliver(const Net &n, int i, int grid_x, cudaStream_t st);
+// hubs: the hub rows in device memory, null without any
+struct HubRows;
+void launch_deliver(const Net &n, int i, int grid_x, int part_shift, const HubRows *hubs, cudaStream_t st);
 
 void prepare_kernel_attributes();
 void prepare_step_kernel_attributes();

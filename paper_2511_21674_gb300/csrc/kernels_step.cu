@@ -2,6 +2,7 @@
 // signal, spike transmission through the delayed synapses.
 #include <cstddef>
 
+#include "delivery_split.h"
 #include "eprop.h"
 #include "eprop_internal.cuh"
 #include "eprop_launch.h"
@@ -419,14 +420,18 @@ __host__ __device__ constexpr size_t deliver_stage_bytes(bool state) {
 // updates, the gradient of update windows that closed since the synapse's
 // last arrival is added on the fly (read-only).  Arrivals are summed in
 // exact int64 fixed point.
-template <bool ALIF, bool STATE>
-__global__ void __launch_bounds__(256, STATE ? 2 : 4) deliver_kernel(Net n, int i, int part_shift) {
+// HUBS: the network has hub rows (their code in every instance cost networks
+// without them 1 to 4 %).
+template <bool ALIF, bool STATE, bool HUBS>
+__global__ void __launch_bounds__(256, STATE ? 2 : 4) deliver_kernel(Net n, int i, int part_shift,
+                                                                        const HubRows *hubs) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ uint64_t bars[8][kDStages];
     __shared__ StageDesc desc[8][kDStages];
     __shared__ RowInfo info[8][STATE ? kDStages : 1][kMaxDelay + 1];
     __shared__ unsigned long long ev_block;
     __shared__ long long ring_off[kMaxDelay + 1];
+    __shared__ int hub_s[HUBS ? kMaxHubs : 1], hub_w[HUBS ? 8 : 1];
     const int b = blockIdx.y;
     // (cleared below) the list slot of step r + 1 (filled by the next neuron update) was last
     // used RS steps ago; every reader of it has finished: the delivery and
@@ -466,21 +471,51 @@ __global__ void __launch_bounds__(256, STATE ? 2 : 4) deliver_kernel(Net n, int 
     // work items: (spiking row, one of 2^part_shift equal parts of its
     // synapses), dealt round-robin to the warps; a step has about as many
     // spiking rows as there are warps, and whole rows would leave most warps
-    // idle while a few finish a second row (host rule: launch_deliver)
-    int prow = gw;
+    // idle while a few finish a second row (host rule: delivery_part_shift).
+    // Before them the parts of the spiking hub rows, in the same order in
+    // every block.
+    int hub_items = 0, hub_parts = 1;
+    long long hub_len = 0;
+    if (HUBS) {
+        static_assert(kMaxHubs == 256, "one thread per hub row");
+        const int src = (int)threadIdx.x < hubs->n ? hubs->src[threadIdx.x] : -1;
+        const unsigned on = __ballot_sync(0xffffffffu, src >= 0 && bit_at(src_words(n, b, src), n.RW, r));
+        if (lane == 0) hub_w[warp] = __popc(on);
+        __syncthreads();
+        int pos = __popc(on & ((1u << lane) - 1u));
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) pos += hub_w[w];
+            hub_items += hub_w[w];
+        }
+        if ((on >> lane) & 1u) hub_s[pos] = src;
+        hub_parts = hubs->parts;
+        hub_len = hubs->len;
+        hub_items *= hub_parts;
+        __syncthreads();
+    }
+    long long pitem = gw;
+    const long long pitems = hub_items + delivery_items(bs.total, part_shift);
     long long pq = 0, pre = 0;
     int psrc = -1, pfirst = 0;
     RowInfo rinfo;
     unsigned vmask = 0;
     auto next_item = [&]() -> bool {
         while (pq >= pre) {
-            if (prow >= bs.total << part_shift) return false;
-            const int row = prow >> part_shift, part = prow & ((1 << part_shift) - 1);
-            psrc = bucket_entry(n, ids, bs, row);
-            const long long rb = n.row_ptr[psrc], len = n.row_ptr[psrc + 1] - rb;
-            pq = rb + ((len * part) >> part_shift);
-            pre = rb + ((len * (part + 1)) >> part_shift);
-            prow += nw;
+            if (pitem >= pitems) return false;
+            if (HUBS && pitem < hub_items) {
+                psrc = hub_s[(int)pitem / hub_parts];
+                const long long rb = n.row_ptr[psrc], re = n.row_ptr[psrc + 1];
+                pq = rb + (long long)((int)pitem % hub_parts) * kHubPart;
+                pre = min(re, pq + kHubPart);
+            } else {
+                const long long it = pitem - hub_items;
+                const int part = (int)it & ((1 << part_shift) - 1);
+                psrc = bucket_entry(n, ids, bs, (int)(it >> part_shift));
+                const long long rb = n.row_ptr[psrc], len = n.row_ptr[psrc + 1] - rb;
+                pq = rb + delivery_part_begin(len, part, part_shift);
+                pre = HUBS && len > hub_len ? pq : rb + delivery_part_begin(len, part + 1, part_shift);
+            }
+            pitem += nw;
             pfirst = 1;
             if (STATE && pre > pq && lane >= 1 && lane <= n.D)
                 rinfo = row_info(n, src_words(n, b, psrc), n.anchor_t[(long long)b * n.n_src + psrc],
@@ -766,22 +801,15 @@ void launch_pred_apply(const Net &n, int i, cudaStream_t st) {
     pred_apply_kernel<<<n.B, ((n.n_out + 31) / 32) * 32, 0, st>>>(n, i);
 }
 
-void launch_deliver(const Net &n, int i, int grid_x, cudaStream_t st) {
+void launch_deliver(const Net &n, int i, int grid_x, int part_shift, const HubRows *hubs, cudaStream_t st) {
     const dim3 grid(grid_x, n.B);
-    // four parts per row, more on long rows (at least 512 records each): quarter
-    // rows of 10,000 synapses kept 2.1 blocks busy per SM on average but three on
-    // some, and those set the time (scaling network 84.8 -> 72 ms per call; at 1000
-    // synapses per row 4 parts measured best)
-    int ps = 2;
-    while (((long long)n.segs * kSeg >> (ps + 1)) >= 512 && ps < 10) ++ps;
-    if (n.has_state && !n.dense) {
-        const size_t sm = deliver_stage_bytes(true) * 8 * kDStages;
-        if (n.alif) launch_pdl(deliver_kernel<true, true>, grid, dim3(256), sm, st, n, i, ps);
-        else launch_pdl(deliver_kernel<false, true>, grid, dim3(256), sm, st, n, i, ps);
-    } else {
-        const size_t sm = deliver_stage_bytes(false) * 8 * kDStages;
-        launch_pdl(deliver_kernel<false, false>, grid, dim3(256), sm, st, n, i, ps);
-    }
+    const size_t sm = deliver_stage_bytes(n.has_state && !n.dense) * 8 * kDStages;
+    auto go = [&](auto *with, auto *without) {
+        launch_pdl(hubs ? with : without, grid, dim3(256), sm, st, n, i, part_shift, hubs);
+    };
+    if (!(n.has_state && !n.dense)) go(deliver_kernel<false, false, true>, deliver_kernel<false, false, false>);
+    else if (n.alif) go(deliver_kernel<true, true, true>, deliver_kernel<true, true, false>);
+    else go(deliver_kernel<false, true, true>, deliver_kernel<false, true, false>);
 }
 
 int persistent_blocks(int sm_count) {
@@ -807,9 +835,12 @@ cudaError_t launch_persistent_steps(const Net &n, int T, GridBar *gb, int blocks
 void prepare_step_kernel_attributes() {
     const int sm = (int)(deliver_stage_bytes(true) * 8 * kDStages);
     const int sm0 = (int)(deliver_stage_bytes(false) * 8 * kDStages);
-    cudaFuncSetAttribute(deliver_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    cudaFuncSetAttribute(deliver_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    cudaFuncSetAttribute(deliver_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm0);
+    cudaFuncSetAttribute(deliver_kernel<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(deliver_kernel<true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(deliver_kernel<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(deliver_kernel<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(deliver_kernel<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm0);
+    cudaFuncSetAttribute(deliver_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm0);
 }
 
 }  // namespace eprop

@@ -4,10 +4,12 @@
 #pragma once
 #include <stdint.h>
 
+#ifndef EPROP_HD
 #ifdef __CUDACC__
 #define EPROP_HD __host__ __device__ __forceinline__
 #else
 #define EPROP_HD inline
+#endif
 #endif
 
 namespace eprop {
