@@ -464,9 +464,12 @@ __global__ void __launch_bounds__(BT, 1) sample_steps_kernel(Net n, int i0, int 
                     n.y_rec[((long long)b * T + (i - 1)) * K + k] = y;
                 }
                 // outside the learning window E and the loss are zero times
-                // finite values
+                // values that are finite while y, the target and their
+                // differences are (a target of NaN where the window is closed
+                // gives NaN, as in the per-step kernels)
                 float E = 0.f;
-                bool zero = win == 0 && fabsf(y) < INFINITY;
+                constexpr float kBig = 8.5e37f;      // below 2^126
+                bool zero = win == 0 && fabsf(y) < kBig && fabsf(tgt) < kBig;
                 zero = __all_sync(0xffffffffu, zero);
                 if (sh.KR > 1) {
                     bar_sync(3, RT);
