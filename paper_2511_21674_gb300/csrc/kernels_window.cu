@@ -1100,6 +1100,17 @@ float G[kB];
 // Measured (batch 64, 2512 rows, 5e7 arrivals): one warp per row with FP64
 // sums and a four-float table 705 us; this form 94 us; batch 32 of 2200
 // steps, 140 rows: 2063 -> 74 us.
+// A pair that has left FP32's range (or met an infinity: inf - inf is NaN) is
+// formed again in FP64 from the spike bits.
+__device__ __noinline__ float batched_sum_f64(const Net n, int src, int j, int d) {
+    double G = 0.0;
+    for (int b = 0; b < n.B; ++b)
+        for_each_spike(src_words_c(n, b, src), n.RW, 1, n.T - d, [&](int st) {
+            G += (double)n.qp[((long long)b * n.U + (st + d - 1)) * n.n_rec + j];
+        });
+    return (float)G;
+}
+
 constexpr int kTbThreads = 256;
 constexpr int kTbCap = 32 * kTbThreads;          // spikes listed: at least one round of words
 __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool plain) {
@@ -1211,7 +1222,8 @@ __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool p
             }
             if (slice == 0 && td != 0u) {
                 const long long q = q0 + qi;
-                const float G = hi + lo;
+                float G = hi + lo;
+                if (!plain && !(fabsf(G) < INFINITY)) G = batched_sum_f64(n, src, j, d);
                 const float w0 = n.w[q];
                 const float wn = window_update(n, q, w0, G);
                 if (!n.adam) n.w[q] = wn;
@@ -1238,11 +1250,15 @@ __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool p
 // since the sample's start has a zero state and no arrival: it is skipped,
 // which leaves most input channels of a sample untouched.  The sum over
 // samples is an FP32 pair with an error-free addition (see the batched form
-// above).  Measured (batch 64, 2512 rows, 4.7e5 synapses, windows of 50 steps,
+// above).  Its terms are scaled by 2^-6 (exact from 2^-120 on; the bits of the
+// sum do not change), so that 64 finite ones cannot leave FP32's range, where
+// the addition's error would be inf - inf; a check per addition cost 2 % of a
+// call.  Measured (batch 64, 2512 rows, 4.7e5 synapses, windows of 50 steps,
 // FP32 traces): one warp per row, FP64 sums 452 us per window; this form 193 us.
 constexpr int kWbRows = 4;
 constexpr int kWbCap = 320;                      // spikes of one row (all samples) listed
 constexpr int kWbThreads = 256;
+constexpr float kWbScale = 1.0f / kBatchWindowMax;
 static_assert(kWbRows * kBatchWindowMax == kWbThreads, "one thread per (row, sample)");
 
 template <bool ALIF, int TB, bool GEN>
@@ -1369,7 +1385,7 @@ __global__ void __launch_bounds__(kWbThreads, 2) window_batched_kernel(Net n, in
                     store_trace(n.ebar, qb, ebar, TB);
                     if (ALIF) store_trace(n.epsa, qb, epsa, TB);
                     float e;
-                    two_sum(hi[r], G, hi[r], e);
+                    two_sum(hi[r], kWbScale * G, hi[r], e);
                     lo[r] += e;
                 }
             }
@@ -1393,7 +1409,8 @@ __global__ void __launch_bounds__(kWbThreads, 2) window_batched_kernel(Net n, in
 #pragma unroll
             for (int r = 0; r < kWbRows; ++r) {
                 if (td[r] == 0u) continue;
-                const float Gf = hi[r] + lo[r];
+                // an infinite term leaves NaN in lo
+                const float Gf = (fabsf(hi[r]) < INFINITY ? hi[r] + lo[r] : hi[r]) * (1.0f / kWbScale);
                 if (Gf != 0.f) {
                     const float w = n.w[q[r]];
                     if (GEN) {
