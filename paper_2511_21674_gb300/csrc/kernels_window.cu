@@ -151,6 +151,69 @@ __device__ __forceinline__ float pair_mul(float a, float b) { return a * b; }
 __device__ __forceinline__ float pair_add(float a, float b) { return a + b; }
 __device__ __forceinline__ float pair_float(float a) { return a; }
 
+// The sweep of tables_kernel below in FP64, for one neuron whose pairs left
+// FP32's range (the error of a product or a sum is then inf - inf): values that
+// come back into range are finite, the others the infinity of their sign.
+template <bool ALIF, bool REG, bool STATE>
+__device__ __noinline__ void sweep_f64(const Net n, int b, int j, int a0, int l_lim) {
+    const int U = n.U;
+    const long long N = n.n_rec;
+    const float *psi = n.psi_hist + (long long)b * (U + 1) * N + j;
+    const float *L = n.L_win + (long long)b * U * N + j;
+    const float *Rs = REG ? n.R_win + (long long)b * U * N + j : nullptr;
+    const long long qbase = (long long)b * U * N + j;
+    const double alpha = (double)n.alpha + (double)n.alpha_lo, ke = (double)n.kappa_e + (double)n.kappa_e_lo;
+    const double rho = ALIF ? (double)n.rho + (double)n.rho_lo : 0.0, beta = n.beta_a;
+    double mz = 0, ma = 0, me = 0, ez = 0, ea = 0, ee = 1, az = 0, aa = 1, ae = 0, mb = 0, pn = 0;
+    auto back = [&](double &xz, double &xa, double D, double p) {
+        if (ALIF) {
+            const double g1 = alpha - beta * p, g2 = rho - beta * p;
+            const double z = alpha * xz + p * xa + pn * g1 * D;
+            xa = g2 * xa - beta * pn * g2 * D;
+            xz = z;
+        } else {
+            xz = alpha * xz + alpha * pn * D;
+        }
+    };
+    for (int u = U; u >= 0; --u) {
+        const double p = psi[u * N];
+        if (u < U) {
+            back(mz, ma, REG ? me + mb : me, p);
+            me *= ke;
+            if (REG) mb *= (double)n.beta_reg;
+            if (STATE) {
+                back(ez, ea, ee, p);
+                ee *= ke;
+                if (ALIF) {
+                    back(az, aa, ae, p);
+                    ae *= ke;
+                }
+            }
+        }
+        if (u == 0) break;
+        const int ul = u + n.d_out;
+        if (ul <= l_lim) me += (double)L[(ul - 1) * N];
+        if (REG) mb += (double)Rs[(u - 1) * N];
+        const float Q = (float)(mz + p * (REG ? me + mb : me));
+        const long long q = qbase + (u - 1) * N;
+        if (!STATE) n.qp[q] = Q;
+        else if (ALIF)
+            reinterpret_cast<float4 *>(n.qp)[q] = make_float4(Q, (float)(ez + p * ee), (float)(az + p * ae), 0.f);
+        else reinterpret_cast<float2 *>(n.qp)[q] = make_float2(Q, (float)(ez + p * ee));
+        pn = p;
+    }
+    if (STATE) {
+        const long long cj = ((long long)b * N + j) * n.RC + ((a0 / U) & (n.RC - 1));
+        if (ALIF) {
+            float4 *c = reinterpret_cast<float4 *>(n.coef) + cj * 2;
+            c[0] = make_float4((float)mz, (float)ma, (float)me, (float)az);
+            c[1] = make_float4((float)aa, (float)ez, (float)ea, 0.f);
+        } else {
+            reinterpret_cast<float4 *>(n.coef)[cj] = make_float4((float)mz, (float)me, (float)ez, 0.f);
+        }
+    }
+}
+
 // learning-signal tables: one thread per (sample, neuron).  The window is
 // swept backwards in chunks of steps: the chunk's learning signals L^t =
 // sum_k B_jk E_k^t (Eq. final-gradient; formed for the whole window beforehand
@@ -207,6 +270,7 @@ __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
     R az = zero, aa = one, ae = zero;
     R mb = zero;                               // adjoint of F_beta(e) (regularisation)
     float pn = 0.f;
+    float q_last = 0.f;
     // x -> (A^{u+1})^T x with A^{u+1} from psi^u = p, psi^{u+1} = pn; D =
     // adjoint of e^{u+1} (both filters of the eligibility).  With X = pn D and
     // Y = xa - beta X:  xz' = alpha (xz + X) + p Y,  xa' = (rho - beta p) Y.
@@ -280,6 +344,7 @@ __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
             if (REG) mb = pair_add(mb, Rc[c]);
             const R De = REG ? pair_add(me, mb) : me;        // adjoint of e^u
             const float Q = pair_float(pair_add(mz, pair_mul(De, p)));
+            q_last = Q;
             if (!STATE) {
                 n.qp[qbase + (long long)(u - 1) * N] = Q;
             } else if (ALIF) {
@@ -305,9 +370,14 @@ __global__ void __launch_bounds__(128, 4) tables_kernel(Net n, int i_end) {
         }
     }
     if (!act) return;
+    // an adjoint that is not finite stays so to the end of the sweep, and a
+    // product that was not joins mz one step later: one look at the end
+    const float end = (q_last + pair_float(mz)) + (pair_float(ma) + pair_float(me)) + pair_float(mb);
+    const bool redo = PAIR && !(fabsf(end) < INFINITY);
+    if (redo) sweep_f64<ALIF, REG, STATE>(n, b, j, a0, l_lim);
     // window coefficients: c = (mz, ma, me), Phi rows (ez, ea, .) and (az, aa, .);
     // one set per sample ([B][N][RC])
-    if (STATE) {
+    if (STATE && !redo) {
         const int slot = (a0 / U) & (n.RC - 1);
         const long long cj = ((long long)b * N + j) * n.RC + slot;
         if (ALIF) {
