@@ -14,6 +14,7 @@
 #include "eprop_launch.h"
 #include "eprop_predictor.h"
 #include "predictor_internal.h"
+#include "spike_lists.h"
 
 using eprop::Net;
 
@@ -174,8 +175,9 @@ static eprop_status alloc_window(eprop_net *net, int U, int T) {
     if (net->trace_mode == 3 && U + D > 65536)
         return fail(net, EPROP_EINVAL, "trace_kernel 4 needs update windows of at most 65536 - max_delay steps");
     n.dense = (net->trace_mode == 2 || net->trace_mode == 3) ? 1 : 0;
-    // the readout reads the spike list of the step d_out back
-    n.RS = std::max(net->trace_mode != 1 ? U + D + 1 : 2, c.d_out + 2);
+    n.list_cap = (int)((((S + 255) / 256) + eprop::kBkt - 1) / eprop::kBkt * 256);
+    n.RS = eprop::spike_list_slots(U, D, c.d_out, net->trace_mode != 1, (int)B,
+                                   B * eprop::kBkt * (long long)n.list_cap * 4);
     n.RC = 0;
     if (n.has_state && n.dense) {
         n.RC = 1;                       // only the current window's coefficients
@@ -198,7 +200,6 @@ static eprop_status alloc_window(eprop_net *net, int U, int T) {
         n.field = reinterpret_cast<decltype(n.field)>(p);                        \
     } while (0)
     WA(bits, uint32_t, B * S * n.RW);
-    n.list_cap = (int)((((S + 255) / 256) + eprop::kBkt - 1) / eprop::kBkt * 256);
     WA(list_ids, int, B * n.RS * eprop::kBkt * (long long)n.list_cap);
     WA(list_cnt, int, B * n.RS * eprop::kBkt);
     WA(psi_hist, float, B * (U + 1) * N);
