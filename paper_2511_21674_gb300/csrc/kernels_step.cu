@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(256, STATE ? 2 : 4) deliver_kernel(Net n, int 
         const StageBuf &sb = buf(k);
         // (to the item's end only: parts of short rows hold a few records, and
         // the conversions below run for absent ones too; rows of 30 at 3e6 events
-        // per step 159 -> 133 us)
+        // per step 159 -> 133 us, with one conversion for one record 125)
 #pragma unroll 2
         for (int h = 0; 32 * h < d.n; h += 4) {
             uint32_t td[4];
@@ -603,7 +603,15 @@ __global__ void __launch_bounds__(256, STATE ? 2 : 4) deliver_kernel(Net n, int 
                 }
             }
             long long fx[4];
-            to_fixed(wv, fx);
+            if (d.n - 32 * h > 32) {
+                to_fixed(wv, fx);
+            } else {                             // one record per lane
+                const float w1[1] = {wv[0]};
+                long long f1[1];
+                to_fixed(w1, f1);
+                fx[0] = f1[0];
+                fx[1] = fx[2] = fx[3] = 0;
+            }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (td[u] == 0u) continue;
