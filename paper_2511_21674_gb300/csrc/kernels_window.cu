@@ -1158,8 +1158,8 @@ float G[kB];
 }
 
 // event-driven synapse gradient, batched single-window form (no carried
-// state: each arrival contributes Q(a) independently).  One block per source
-// row: its threads scan the row's spike bits of every sample and compact them
+// state: each arrival contributes Q(a) independently).  One block (or warp) per
+// source row: its threads scan the row's spike bits of every sample and compact them
 // (block scan, so in sample and step order) into a list in shared memory;
 // then each thread owns one synapse (or, on short rows, a share of its
 // spikes) and sums the table entries of the arrivals.  The sum (up to
@@ -1181,17 +1181,29 @@ __device__ __noinline__ float batched_sum_f64(const Net n, int src, int j, int d
     return (float)G;
 }
 
-constexpr int kTbThreads = 256;
-constexpr int kTbCap = 32 * kTbThreads;          // spikes listed: at least one round of words
-__global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool plain) {
-    __shared__ uint32_t sp[kTbCap];              // spike_entry.h
+// G threads serve a row: the block, or, where rows are many and their words
+// few, a warp (eight rows per block; launch_trace_batched).
+// Five blocks per SM: the loads of the four unrolled look-ups need 44 registers
+// (with room for a sixth block, 38, calls of 60,000 neurons x 32 samples took
+// 19.3 instead of 16.9 ms), and the grid is one wave.
+constexpr int kTbThreads = 256, kTbBlocks = 5;
+template <int G>
+__global__ void __launch_bounds__(kTbThreads, kTbBlocks) trace_batched_kernel(Net n, bool plain) {
+    constexpr int kRows = kTbThreads / G;
+    constexpr int kCap = 32 * G;                 // spikes listed: at least one round of words
+    __shared__ uint32_t sp_s[kRows][kCap];       // spike_entry.h
     __shared__ int wsum[kTbThreads / 32];
-    __shared__ float2 red[kTbThreads];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ float2 red[G == 32 ? 1 : kTbThreads];
+    const int tid = threadIdx.x % G, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *sp = sp_s[threadIdx.x / G];
+    auto sync = [] {
+        if constexpr (G == 32) __syncwarp();
+        else __syncthreads();
+    };
     const int U = n.U, N = n.n_rec, T = n.T;
     const int wps = T / 32 + 1;                  // words per sample holding steps 1..T
     const int nwords = n.B * wps;
-    for (int src = blockIdx.x; src < n.n_src; src += gridDim.x) {
+    for (int src = blockIdx.x * kRows + threadIdx.x / G; src < n.n_src; src += gridDim.x * kRows) {
         const long long q0 = n.row_ptr[src];
         const int len = (int)(n.row_ptr[src + 1] - q0);
         if (len == 0) continue;
@@ -1221,25 +1233,29 @@ __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool p
                     const int t = __shfl_up_sync(0xffffffffu, x, o);
                     if (lane >= o) x += t;
                 }
-                __syncthreads();                 // earlier readers of wsum and sp are done
-                if (lane == 31) wsum[warp] = x;
-                __syncthreads();
+                sync();                          // earlier readers of wsum and sp are done
                 int before = 0, all = 0;
+                if constexpr (G == 32) {
+                    all = __shfl_sync(0xffffffffu, x, 31);
+                } else {
+                    if (lane == 31) wsum[warp] = x;
+                    sync();
 #pragma unroll
-                for (int v = 0; v < kTbThreads / 32; ++v) {
-                    if (v < warp) before += wsum[v];
-                    all += wsum[v];
+                    for (int v = 0; v < G / 32; ++v) {
+                        if (v < warp) before += wsum[v];
+                        all += wsum[v];
+                    }
                 }
-                if (ns + all > kTbCap) break;    // (never in the first round)
+                if (ns + all > kCap) break;      // (never in the first round)
                 int pos = ns + before + x - c;
                 while (m) {
                     sp[pos++] = entry_pack(base, b, k * 32 + __ffs(m) - 1, U, T);
                     m &= m - 1;
                 }
                 ns += all;
-                w0 = min(w0 + kTbThreads, w_end);
+                w0 = min(w0 + G, w_end);
             }
-            __syncthreads();
+            sync();
             return w0;
         };
         int next = fill(0);
@@ -1247,12 +1263,12 @@ __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool p
         if (whole && ns == 0) continue;
         // threads per synapse group: the row's synapses, rounded up to warps
         int tc = 32;
-        while (tc < len && tc < kTbThreads) tc <<= 1;
+        while (tc < len && tc < G) tc <<= 1;
         // plain: the FP32 sum in step order, as the work-queue form rounds it (a
         // single-sample network that the automatic choice brings here keeps
         // that form's bits)
-        if (plain) tc = kTbThreads;
-        const int slices = kTbThreads / tc, slice = tid / tc, tq = tid - slice * tc;
+        if (plain) tc = G;
+        const int slices = G / tc, slice = tid / tc, tq = tid - slice * tc;
         for (int qc = 0; qc < len; qc += tc) {
             const int qi = qc + tq;
             const uint32_t td = qi < len ? n.tgt_d[q0 + qi] : 0u;
@@ -1278,9 +1294,9 @@ __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool p
                 if (next >= nwords) break;
                 next = fill(next);
             }
-            if (slices > 1) {
+            if (G > 32 && slices > 1) {
                 red[tid] = make_float2(hi, lo);
-                __syncthreads();
+                sync();
                 if (slice == 0)
                     for (int v = 1; v < slices; ++v) {
                         const float2 o = red[v * tc + tq];
@@ -1288,16 +1304,16 @@ __global__ void __launch_bounds__(kTbThreads) trace_batched_kernel(Net n, bool p
                         two_sum(hi, o.x, hi, e);
                         lo += e + o.y;
                     }
-                __syncthreads();
+                sync();
             }
             if (slice == 0 && td != 0u) {
                 const long long q = q0 + qi;
-                float G = hi + lo;
-                if (!plain && !(fabsf(G) < INFINITY)) G = batched_sum_f64(n, src, j, d);
+                float g = hi + lo;
+                if (!plain && !(fabsf(g) < INFINITY)) g = batched_sum_f64(n, src, j, d);
                 const float w0 = n.w[q];
-                const float wn = window_update(n, q, w0, G);
+                const float wn = window_update(n, q, w0, g);
                 if (!n.adam) n.w[q] = wn;
-                if (n.record_grad) n.grad[q] += n.inv_B * G;
+                if (n.record_grad) n.grad[q] += n.inv_B * g;
             }
         }
     }
@@ -1996,9 +2012,24 @@ void launch_window_batched(const Net &n, int i_end, int sm_count, cudaStream_t s
 #undef EPROP_WB
 }
 
+// Whether the batched kernels give a source row to a warp or to a block (or a
+// block four rows).  A block per row pays its scan and barriers for every row
+// and keeps few rows in flight, which many short rows feel; a warp per row leaves
+// SMs idle on few rows and walks a long one alone.  Measured, block / warp:
+// ms per call of 100 steps, single window: 1e5 rows of 30 4.21 / 3.94; 1e5 rows of
+// 1000, 2 samples 7.67 / 7.51; 20,000 rows of 1000, 8 samples 2.70 / 2.80; 2512 rows of
+// 200, 8 samples (200 steps) 0.462 / 0.478.
+static bool row_per_warp(const Net &n, int sm_count) {
+    const long long mean = n.nnz / (n.n_src > 0 ? n.n_src : 1);
+    return n.n_src >= 48LL * sm_count && (mean <= 256 || n.n_src >= 512LL * sm_count);
+}
+
 void launch_trace_batched(const Net &n, bool plain, int sm_count, cudaStream_t st) {
-    const int blocks = n.n_src < 6 * sm_count ? n.n_src : 6 * sm_count;
-    trace_batched_kernel<<<blocks, kTbThreads, 0, st>>>(n, plain);
+    const bool warps = row_per_warp(n, sm_count);
+    const int rows = warps ? kTbThreads / 32 : 1, want = (n.n_src + rows - 1) / rows;
+    const int blocks = want < kTbBlocks * sm_count ? want : kTbBlocks * sm_count;
+    if (warps) trace_batched_kernel<32><<<blocks, kTbThreads, 0, st>>>(n, plain);
+    else trace_batched_kernel<kTbThreads><<<blocks, kTbThreads, 0, st>>>(n, plain);
 }
 
 void launch_readout_weights(const Net &n, int i_end, cudaStream_t st) {
