@@ -1341,22 +1341,38 @@ __global__ void __launch_bounds__(kTbThreads, kTbBlocks) trace_batched_kernel(Ne
 // the addition's error would be inf - inf; a check per addition cost 2 % of a
 // call.  Measured (batch 64, 2512 rows, 4.7e5 synapses, windows of 50 steps,
 // FP32 traces): one warp per row, FP64 sums 452 us per window; this form 193 us.
+//
+// R: rows of a group.  The block is one group of four rows, or, where rows are
+// many and short (row_per_warp), eight groups (a warp each) of one row: a block
+// per four rows of 30 is bound by latency, look-ups one after another at 16 warps
+// per SM, which 32 warps of one row hide.
 constexpr int kWbRows = 4;
-constexpr int kWbCap = 320;                      // spikes of one row (all samples) listed
 constexpr int kWbThreads = 256;
 constexpr float kWbScale = 1.0f / kBatchWindowMax;
 static_assert(kWbRows * kBatchWindowMax == kWbThreads, "one thread per (row, sample)");
 
-template <bool ALIF, int TB, bool GEN>
-__global__ void __launch_bounds__(kWbThreads, 2) window_batched_kernel(Net n, int i_end) {
+template <bool ALIF, int TB, bool GEN, int R>
+__global__ void __launch_bounds__(kWbThreads, R == 1 ? 4 : 2) window_batched_kernel(Net n, int i_end) {
     constexpr unsigned kFull = 0xffffffffu;
-    __shared__ float zb[kWbRows][kBatchWindowMax][kMaxDelay + 1];
-    __shared__ int sp[kWbRows][kWbCap];
-    __shared__ int soff[kWbRows][kBatchWindowMax + 1];
+    constexpr int kGroup = R == 1 ? 32 : kWbThreads;               // threads of a group
+    constexpr int kGroups = kWbThreads / kGroup, kSlots = R * kBatchWindowMax / kGroup;
+    constexpr int kWbCap = R == 1 ? 256 : 320;   // spikes of one row (all samples) listed
+    __shared__ float zb_s[kGroups][R][kBatchWindowMax][kMaxDelay + 1];
+    __shared__ int sp_s[kGroups][R][kWbCap];
+    __shared__ int soff_s[kGroups][R][kBatchWindowMax + 1];
     __shared__ int warp_n[kWbThreads / 32];
-    __shared__ uint8_t active[kWbRows][kBatchWindowMax];
-    __shared__ float2 red[kWbRows][kWbThreads];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ uint8_t active_s[kGroups][R][kBatchWindowMax];
+    __shared__ float2 red[R][R == 1 ? 1 : kWbThreads];
+    const int group = threadIdx.x / kGroup, tid = threadIdx.x % kGroup;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto &zb = zb_s[group];
+    auto &sp = sp_s[group];
+    auto &soff = soff_s[group];
+    auto &active = active_s[group];
+    auto sync = [] {
+        if constexpr (R == 1) __syncwarp();
+        else __syncthreads();
+    };
     const int U = n.U, N = n.n_rec, B = n.B, D = n.D;
     const int r_end = run_step_w(n, i_end);
     const int a0 = r_end - U;
@@ -1364,70 +1380,85 @@ __global__ void __launch_bounds__(kWbThreads, 2) window_batched_kernel(Net n, in
     const float step = n.lr * n.inv_B;
     const long long nnz = n.nnz;
     const long long cstride = (long long)N * n.RC;
-    const int groups = (n.n_src + kWbRows - 1) / kWbRows;
-    for (int g = blockIdx.x; g < groups; g += gridDim.x) {
-        const int src0 = g * kWbRows;
-        __syncthreads();                         // the previous group's lists are read
-        // this thread's (row, sample): spikes of the window and activity
-        const int tr = tid / kBatchWindowMax, tb = tid % kBatchWindowMax;
-        const bool pair_in = src0 + tr < n.n_src && tb < B;
-        const uint32_t *words = pair_in ? src_words_c(n, tb, src0 + tr) : nullptr;
-        int cnt = 0;
-        if (pair_in && s_lo <= s_hi) for_each_spike(words, n.RW, s_lo, s_hi, [&](int) { ++cnt; });
-        int x = cnt;
+    const int groups = (n.n_src + R - 1) / R;
+    for (int g = blockIdx.x * kGroups + group; g < groups; g += gridDim.x * kGroups) {
+        const int src0 = g * R;
+        sync();                                  // the previous group's lists are read
+        // this thread's (row, sample), two of them in a warp: spikes of the
+        // window and activity
+        int cnt[kSlots], x[kSlots];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, x, o);
-            if (lane >= o) x += t;
-        }
-        if (lane == 31) warp_n[warp] = x;
-        if (pair_in) {
-            const long long sb = (long long)tb * n.n_src + src0 + tr;
-            const int at = n.anchor_t[sb];
-            active[tr][tb] = cnt > 0 || at != kNoSpike;
-            if (active[tr][tb])
-                for (int d = 1; d <= D; ++d)
-                    zb[tr][tb][d] = row_info(n, words, at, n.anchor_z[sb], a0, d, false).zbar_a0;
-        } else {
-            active[tr][tb] = 0;
-        }
-        __syncthreads();
-        // a row's 64 samples are two warps
-        const int pos0 = x - cnt + ((warp & 1) ? warp_n[warp - 1] : 0);
-        soff[tr][tb] = pos0;
-        if (tb == kBatchWindowMax - 1) soff[tr][kBatchWindowMax] = pos0 + cnt;
-        if (cnt && warp_n[warp & ~1] + warp_n[warp | 1] <= kWbCap) {
-            int pos = pos0;
-            for_each_spike(words, n.RW, s_lo, s_hi, [&](int st) { sp[tr][pos++] = st; });
-        }
-        __syncthreads();
-        int len[kWbRows], maxlen = 0;
-        bool listed[kWbRows];
+        for (int h = 0; h < kSlots; ++h) {
+            const int tr = R == 1 ? 0 : tid / kBatchWindowMax, tb = (tid + 32 * h) % kBatchWindowMax;
+            const bool pair_in = src0 + tr < n.n_src && tb < B;
+            const uint32_t *words = pair_in ? src_words_c(n, tb, src0 + tr) : nullptr;
+            cnt[h] = 0;
+            if (pair_in && s_lo <= s_hi) for_each_spike(words, n.RW, s_lo, s_hi, [&](int) { ++cnt[h]; });
+            x[h] = cnt[h];
 #pragma unroll
-        for (int r = 0; r < kWbRows; ++r) {
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(kFull, x[h], o);
+                if (lane >= o) x[h] += t;
+            }
+            if (pair_in) {
+                const long long sb = (long long)tb * n.n_src + src0 + tr;
+                const int at = n.anchor_t[sb];
+                active[tr][tb] = cnt[h] > 0 || at != kNoSpike;
+                if (active[tr][tb])
+                    for (int d = 1; d <= D; ++d)
+                        zb[tr][tb][d] = row_info(n, words, at, n.anchor_z[sb], a0, d, false).zbar_a0;
+            } else {
+                active[tr][tb] = 0;
+            }
+        }
+        // spikes of the row's first 32 samples, and of all
+        int first, row_n;
+        if (R == 1) {
+            first = __shfl_sync(kFull, x[0], 31);
+            row_n = first + __shfl_sync(kFull, x[kSlots - 1], 31);
+        } else {                                 // a row's 64 samples are two warps
+            if (lane == 31) warp_n[warp] = x[0];
+            sync();
+            first = warp_n[warp & ~1];
+            row_n = first + warp_n[warp | 1];
+        }
+#pragma unroll
+        for (int h = 0; h < kSlots; ++h) {
+            const int tr = R == 1 ? 0 : tid / kBatchWindowMax, tb = (tid + 32 * h) % kBatchWindowMax;
+            int pos = x[h] - cnt[h] + (tb >= 32 ? first : 0);
+            soff[tr][tb] = pos;
+            if (tb == kBatchWindowMax - 1) soff[tr][kBatchWindowMax] = pos + cnt[h];
+            if (cnt[h] && row_n <= kWbCap)
+                for_each_spike(src_words_c(n, tb, src0 + tr), n.RW, s_lo, s_hi, [&](int st) { sp[tr][pos++] = st; });
+        }
+        sync();
+        int len[R], maxlen = 0;
+        bool listed[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
             const bool in = src0 + r < n.n_src;
             len[r] = in ? (int)(n.row_ptr[src0 + r + 1] - n.row_ptr[src0 + r]) : 0;
             listed[r] = soff[r][kBatchWindowMax] <= kWbCap;
             maxlen = max(maxlen, len[r]);
         }
         int tc = 32;
-        while (tc < maxlen && tc < kWbThreads) tc <<= 1;
-        const int slices = kWbThreads / tc, slice = tid / tc, tq = tid - slice * tc;
+        while (tc < maxlen && tc < kGroup) tc <<= 1;
+        const int slices = kGroup / tc, slice = tid / tc, tq = tid - slice * tc;
         for (int qc = 0; qc < maxlen; qc += tc) {
-            long long q[kWbRows];
-            uint32_t td[kWbRows];
-            float hi[kWbRows], lo[kWbRows];
+            long long q[R];
+            uint32_t td[R];
+            float hi[R], lo[R];
 #pragma unroll
-            for (int r = 0; r < kWbRows; ++r) {
+            for (int r = 0; r < R; ++r) {
                 q[r] = (src0 + r < n.n_src ? n.row_ptr[src0 + r] : 0) + qc + tq;
                 td[r] = qc + tq < len[r] ? n.tgt_d[q[r]] : 0u;
                 hi[r] = lo[r] = 0.f;
             }
             for (int b = slice; b < B; b += slices) {
-                float eb[kWbRows], ep[kWbRows];
-                bool use[kWbRows];
+                float eb[R], ep[R];
+                bool use[R];
 #pragma unroll
-                for (int r = 0; r < kWbRows; ++r) {
+                for (int r = 0; r < R; ++r) {
                     use[r] = td[r] != 0u && active[r][b];
                     const long long qb = (long long)b * nnz + q[r];
                     eb[r] = use[r] ? load_trace(n.ebar, qb, TB) : 0.f;
@@ -1437,7 +1468,7 @@ __global__ void __launch_bounds__(kWbThreads, 2) window_batched_kernel(Net n, in
                 int jc = -1;
                 const long long qa = ((long long)b * U - a0 - 1) * N;   // table index qa + a * N + j
 #pragma unroll
-                for (int r = 0; r < kWbRows; ++r) {
+                for (int r = 0; r < R; ++r) {
                     if (!use[r]) continue;
                     const int j = (int)(td[r] & 0xFFFFFFu), dl = (int)(td[r] >> 24);
                     if (j != jc) {
@@ -1475,13 +1506,13 @@ __global__ void __launch_bounds__(kWbThreads, 2) window_batched_kernel(Net n, in
                     lo[r] += e;
                 }
             }
-            if (slices > 1) {
+            if (R > 1 && slices > 1) {
 #pragma unroll
-                for (int r = 0; r < kWbRows; ++r) red[r][tid] = make_float2(hi[r], lo[r]);
-                __syncthreads();
+                for (int r = 0; r < R; ++r) red[r][tid] = make_float2(hi[r], lo[r]);
+                sync();
                 if (slice == 0) {
 #pragma unroll
-                    for (int r = 0; r < kWbRows; ++r)
+                    for (int r = 0; r < R; ++r)
                         for (int v = 1; v < slices; ++v) {
                             const float2 o = red[r][v * tc + tq];
                             float e;
@@ -1489,11 +1520,11 @@ __global__ void __launch_bounds__(kWbThreads, 2) window_batched_kernel(Net n, in
                             lo[r] += e + o.y;
                         }
                 }
-                __syncthreads();
+                sync();
             }
             if (slice != 0) continue;
 #pragma unroll
-            for (int r = 0; r < kWbRows; ++r) {
+            for (int r = 0; r < R; ++r) {
                 if (td[r] == 0u) continue;
                 // an infinite term leaves NaN in lo
                 const float Gf = (fabsf(hi[r]) < INFINITY ? hi[r] + lo[r] : hi[r]) * (1.0f / kWbScale);
@@ -1992,13 +2023,33 @@ void launch_window_pass(const Net &n, int i_end, int grid_x, int grid_idle, cuda
 #undef EPROP_PASS
 }
 
+// Whether the batched kernels give a source row to a warp or to a block (or a
+// block four rows).  A block per row pays its scan and barriers for every row
+// and keeps few rows in flight, which many short rows feel; a warp per row leaves
+// SMs idle on few rows and walks a long one alone.  Measured, block / warp:
+// ms per call of 100 steps, single window: 1e5 rows of 30 4.21 / 3.94; 1e5 rows of
+// 1000, 2 samples 7.67 / 7.51; 20,000 rows of 1000, 8 samples 2.70 / 2.80; 2512 rows of
+// 200, 8 samples (200 steps) 0.462 / 0.478.  Windows of 50 steps: 60,000 rows of 30, 8
+// samples 30.5 / 28.3; 1e5 rows of 1000, 2 samples 9.76 / 8.86; 20,000 rows of 1000, 8 samples
+// 3.09 / 3.18; 2512 rows of 200, 8 samples 0.676 / 0.768.
+static bool row_per_warp(const Net &n, int sm_count) {
+    const long long mean = n.nnz / (n.n_src > 0 ? n.n_src : 1);
+    return n.n_src >= 48LL * sm_count && (mean <= 256 || n.n_src >= 512LL * sm_count);
+}
+
 void launch_window_batched(const Net &n, int i_end, int sm_count, cudaStream_t st) {
-    int blocks = (n.n_src + kWbRows - 1) / kWbRows;
+    const bool warps = row_per_warp(n, sm_count);
+    const int rows = warps ? kWbThreads / 32 : kWbRows;
+    int blocks = (n.n_src + rows - 1) / rows;
     if (blocks > 8 * sm_count) blocks = 8 * sm_count;
-#define EPROP_WB(A, T)                                                                                   \
-    do {                                                                                                 \
-        if (n.adam || n.sign_mask) window_batched_kernel<A, T, true><<<blocks, kWbThreads, 0, st>>>(n, i_end);  \
-        else window_batched_kernel<A, T, false><<<blocks, kWbThreads, 0, st>>>(n, i_end);                       \
+    auto go = [&](auto *warp_rows, auto *block_rows) {
+        if (warps) warp_rows<<<blocks, kWbThreads, 0, st>>>(n, i_end);
+        else block_rows<<<blocks, kWbThreads, 0, st>>>(n, i_end);
+    };
+#define EPROP_WB(A, T)                                                                                             \
+    do {                                                                                                           \
+        if (n.adam || n.sign_mask) go(window_batched_kernel<A, T, true, 1>, window_batched_kernel<A, T, true, kWbRows>);    \
+        else go(window_batched_kernel<A, T, false, 1>, window_batched_kernel<A, T, false, kWbRows>);               \
     } while (0)
 #define EPROP_WB_T(A)                                  \
     do {                                               \
@@ -2010,18 +2061,6 @@ void launch_window_batched(const Net &n, int i_end, int sm_count, cudaStream_t s
     else EPROP_WB_T(false);
 #undef EPROP_WB_T
 #undef EPROP_WB
-}
-
-// Whether the batched kernels give a source row to a warp or to a block (or a
-// block four rows).  A block per row pays its scan and barriers for every row
-// and keeps few rows in flight, which many short rows feel; a warp per row leaves
-// SMs idle on few rows and walks a long one alone.  Measured, block / warp:
-// ms per call of 100 steps, single window: 1e5 rows of 30 4.21 / 3.94; 1e5 rows of
-// 1000, 2 samples 7.67 / 7.51; 20,000 rows of 1000, 8 samples 2.70 / 2.80; 2512 rows of
-// 200, 8 samples (200 steps) 0.462 / 0.478.
-static bool row_per_warp(const Net &n, int sm_count) {
-    const long long mean = n.nnz / (n.n_src > 0 ? n.n_src : 1);
-    return n.n_src >= 48LL * sm_count && (mean <= 256 || n.n_src >= 512LL * sm_count);
 }
 
 void launch_trace_batched(const Net &n, bool plain, int sm_count, cudaStream_t st) {
