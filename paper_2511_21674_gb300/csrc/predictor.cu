@@ -90,8 +90,7 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], 
 // (g+8, ..), (g, 2t+8..), (g+8, 2t+8..); B (2t..2t+1, g), (2t+8.., g); C (g,
 // 2t..2t+1), (g+8, 2t..2t+1).
 constexpr int kChunkK = 64, kChunkN = 256;
-constexpr int kMlpThreads = 256;
-constexpr int kStageElems = kChunkN * (kChunkK + 8);     // >= kChunkK * (kChunkN + 8)
+constexpr int kMlpThreads = 256, kNarrowThreads = 64;
 
 struct Mlp {
     int rows, I, H, K, ldX, ldH, ldK, stages;
@@ -103,20 +102,38 @@ struct Mlp {
 };
 
 __host__ __device__ inline int pad16(int x) { return (x + 15) & ~15; }
+// A ring stage holds 64 rows of a layer's columns or, backward, as many rows of
+// 64 columns; narrow networks need few columns (and many blocks then share an SM).
+__host__ __device__ inline int mlp_cols(int H, int K) {
+    const int c = ((H > K ? H : K) + 31) & ~31;
+    return c < kChunkN ? c : kChunkN;
+}
+__host__ __device__ inline int mlp_stage(int H, int K) {
+    const int c = mlp_cols(H, K), fwd = kChunkK * (c + 8), bwd = c * (kChunkK + 8);
+    return fwd > bwd ? fwd : bwd;
+}
+// The inputs' tile is dead once the first layer is done: the second layer's
+// output takes its place.  (Not where its rows have padding columns, which have
+// to stay zero.)
+__host__ __device__ inline bool mlp_alias(int H) { return H % 16 == 0; }
 static size_t mlp_smem(const Mlp &a, int MT, bool train) {
-    const size_t row = (size_t)(pad16(a.I) + 8) + 2 * (size_t)(pad16(a.H) + 8) + (train ? pad16(a.K) + 8 : 0);
-    return (row * 16 * MT + (size_t)a.stages * kStageElems) * sizeof(bf16);
+    const size_t x = (size_t)(pad16(a.I) + 8), h = (size_t)(pad16(a.H) + 8);
+    const size_t row = (mlp_alias(a.H) ? std::max(x, h) : x + h) + h + (train ? pad16(a.K) + 8 : 0);
+    return (row * 16 * MT + (size_t)a.stages * mlp_stage(a.H, a.K)) * sizeof(bf16);
 }
 
-template <int MT, bool TRAIN>
-__global__ void __launch_bounds__(kMlpThreads) mlp_kernel(Mlp a) {
+template <int MT, bool TRAIN, int NT = kMlpThreads>
+__global__ void __launch_bounds__(NT) mlp_kernel(Mlp a) {
     extern __shared__ __align__(16) unsigned char pred_sm[];
-    __shared__ float red[kMlpThreads / 32];
+    __shared__ float red[NT / 32];
     const int SX = pad16(a.I) + 8, SH = pad16(a.H) + 8, SK = pad16(a.K) + 8;
     constexpr int R = 16 * MT;
     bf16 *ring = reinterpret_cast<bf16 *>(pred_sm);
-    bf16 *Xs = ring + (size_t)a.stages * kStageElems;
-    bf16 *P1 = Xs + R * SX, *P2 = P1 + R * SH, *dYs = P2 + R * SH;
+    const int stage_n = mlp_stage(a.H, a.K), ldS = mlp_cols(a.H, a.K) + 8;
+    bf16 *Xs = ring + (size_t)a.stages * stage_n;
+    const bool alias = mlp_alias(a.H);
+    bf16 *P1 = Xs + R * (alias ? max(SX, SH) : SX), *P2 = alias ? Xs : P1 + R * SH;
+    bf16 *dYs = alias ? P1 + R * SH : P2 + R * SH;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int r0 = blockIdx.x * R;
     // phases: 0..2 the layers, 3 dA2 = dY W3^T, 4 dA1 = dA2 W2^T
@@ -143,19 +160,33 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_kernel(Mlp a) {
                 const bf16 *W = p.ph == 0 ? a.W1 : p.ph == 1 ? a.W2 : a.W3;
                 const int ld = p.ph == 2 ? a.ldK : a.ldH;
                 const int pieces = (min(kChunkN, N - p.n0) + 31) / 32 * 4;      // of 8 columns
-                for (int q = tid; q < kChunkK * pieces; q += kMlpThreads) {
-                    const int k = q / pieces, c = (q - k * pieces) * 8;
+                auto piece = [&](int k, int c) {
                     const bool in = p.k0 + k < Kd && p.n0 + c < ld;
-                    cp16(st + k * (kChunkN + 8) + c, in ? W + (size_t)(p.k0 + k) * ld + p.n0 + c : W, in);
+                    cp16(st + k * ldS + c, in ? W + (size_t)(p.k0 + k) * ld + p.n0 + c : W, in);
+                };
+                // a full chunk without divisions: with two per copy, 1024-1024-1024
+                // took 395 us for one row (192 chunks), now 263
+                if (pieces == kChunkN / 8) {
+#pragma unroll
+                    for (int i = 0; i < kChunkK * kChunkN / 8 / NT; ++i)
+                        piece((tid >> 5) + i * (NT / 32), (tid & 31) * 8);
+                } else {
+                    for (int q = tid; q < kChunkK * pieces; q += NT) piece(q / pieces, q % pieces * 8);
                 }
             } else {
                 const bf16 *W = p.ph == 3 ? a.W3 : a.W2;
                 const int ld = p.ph == 3 ? a.ldK : a.ldH;
                 const int pieces = min(kChunkK, pad16(Kd) - p.k0) / 8;
-                for (int q = tid; q < kChunkN * pieces; q += kMlpThreads) {
-                    const int nn = q / pieces, c = (q - nn * pieces) * 8;
+                const int rows = (min(kChunkN, N - p.n0) + 31) & ~31;
+                auto piece = [&](int nn, int c) {
                     const bool in = p.n0 + nn < N && p.k0 + c < ld;
                     cp16(st + nn * (kChunkK + 8) + c, in ? W + (size_t)(p.n0 + nn) * ld + p.k0 + c : W, in);
+                };
+                if (pieces == kChunkK / 8) {
+#pragma unroll 8
+                    for (int nn = tid >> 3; nn < rows; nn += NT / 8) piece(nn, (tid & 7) * 8);
+                } else {
+                    for (int q = tid; q < rows * pieces; q += NT) piece(q / pieces, q % pieces * 8);
                 }
             }
         }
@@ -163,18 +194,22 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_kernel(Mlp a) {
     };
     Pos lp{0, 0, 0};
     for (int q = 0; q < a.stages - 1; ++q) {
-        load(lp, ring + (size_t)q * kStageElems);
+        load(lp, ring + (size_t)q * stage_n);
         if (lp.ph < kPhases) advance(lp);
     }
     // activation tiles: padding columns and rows past the end stay zero
-    for (int q = tid; q < R * (2 * SH + (TRAIN ? SK : 0)) / 2; q += kMlpThreads) reinterpret_cast<uint32_t *>(P1)[q] = 0u;
-    for (int q = tid; q < R * SX; q += kMlpThreads) {
-        const int m = q / SX, c = q - m * SX;
-        float v = 0.f;
-        if (r0 + m < a.rows && c < a.I) v = a.x[(size_t)(r0 + m) * a.I + c] * a.scale[c];
-        const bf16 h = __float2bfloat16_rn(v);
-        Xs[q] = h;
-        if (r0 + m < a.rows && c < a.ldX) a.Xh[(size_t)(r0 + m) * a.ldX + c] = h;
+    const int tiles_n = R * ((alias ? SH : 2 * SH) + (TRAIN ? SK : 0)) / 2;
+    for (int q = tid; q < tiles_n; q += NT) reinterpret_cast<uint32_t *>(P1)[q] = 0u;
+#pragma unroll 4
+    for (int m = warp; m < R; m += NT / 32) {
+        const bool row = r0 + m < a.rows;
+        const float *x = a.x + (size_t)(row ? r0 + m : 0) * a.I;
+        bf16 *xh = a.Xh + (size_t)(row ? r0 + m : 0) * a.ldX;
+        for (int c = lane; c < SX; c += 32) {
+            const bf16 h = __float2bfloat16_rn(row && c < a.I ? x[c] * a.scale[c] : 0.f);
+            Xs[m * SX + c] = h;
+            if (row && c < a.ldX) xh[c] = h;
+        }
     }
     float sq = 0.f;
     float acc[MT][4][4];
@@ -186,10 +221,10 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_kernel(Mlp a) {
         __syncthreads();                 // chunk c is there, chunk c - 1 and its tiles are done
         {
             const int q = c + a.stages - 1;
-            load(lp, ring + (size_t)(q % a.stages) * kStageElems);
+            load(lp, ring + (size_t)(q % a.stages) * stage_n);
             if (lp.ph < kPhases) advance(lp);
         }
-        const bf16 *st = ring + (size_t)(c % a.stages) * kStageElems;
+        const bf16 *st = ring + (size_t)(c % a.stages) * stage_n;
         const int N = ndim(p.ph), Kd = kdim(p.ph);
         const int nb = p.n0 + warp * 32;
         const bool last = p.k0 + kChunkK >= Kd;
@@ -215,7 +250,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_kernel(Mlp a) {
                 for (int h = 0; h < 2; ++h) {
                     const int nl = warp * 32 + h * 16 + (mt >> 1) * 8;
                     const int kl = ks * 16 + (mt & 1) * 8;
-                    if (p.ph < 3) ldm4t(bfr[h], st + (kl + lr) * (kChunkN + 8) + nl);
+                    if (p.ph < 3) ldm4t(bfr[h], st + (kl + lr) * ldS + nl);
                     else ldm4(bfr[h], st + (nl + lr) * (kChunkK + 8) + kl);
                 }
 #pragma unroll
@@ -280,7 +315,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_kernel(Mlp a) {
         __syncthreads();
         if (tid == 0) {
             float s = 0.f;
-            for (int w = 0; w < kMlpThreads / 32; ++w) s += red[w];
+            for (int w = 0; w < NT / 32; ++w) s += red[w];
             a.lpart[blockIdx.x] = s;
         }
     }
@@ -630,14 +665,27 @@ static int issue_mlp(eprop_predictor *p, const float *x, const float *e, int row
     a.inv = 1.0f / (float)rows;
     const bool train = e != nullptr;
     // 32-row tiles once 16-row tiles fill the SMs; four ring stages where they
-    // fit (two at n_in = hidden = n_out = 1024 in training)
+    // fit; of several waves of tiles two blocks share an SM where two stages
+    // allow it (65,536 rows of 74-256-10: inference 619 -> 448 us).  Narrow
+    // layers keep one or two of the eight warps busy: many rows of them run in
+    // blocks of two warps, many to an SM (65,536 rows of 74-64-10: 415 -> 266 us)
     a.stages = 4;
-    int mt = rows > 16 * p->sm_count ? 2 : 1;
+    const int cols = mlp_cols(a.H, a.K);
+    const bool narrow = cols <= kNarrowThreads && rows > 32 * p->sm_count;
+    int mt = rows > 16 * p->sm_count && cols > 128 ? 2 : 1;
     if (mlp_smem(a, mt, train) > (size_t)kMlpSmemMax) mt = 1;
-    while (a.stages > 2 && mlp_smem(a, mt, train) > (size_t)kMlpSmemMax) --a.stages;
     const int tiles = (rows + 16 * mt - 1) / (16 * mt);
+    while (a.stages > 2 && mlp_smem(a, mt, train) > (size_t)kMlpSmemMax) --a.stages;
+    Mlp two = a;
+    two.stages = 2;
+    if (narrow) a.stages = 2;
+    else if (tiles > p->sm_count && mlp_smem(two, mt, train) <= (size_t)kMlpSmemMax / 2)
+        while (mlp_smem(a, mt, train) > (size_t)kMlpSmemMax / 2) --a.stages;
     const size_t sm = mlp_smem(a, mt, train);
-    if (train) {
+    if (narrow) {
+        if (train) mlp_kernel<1, true, kNarrowThreads><<<tiles, kNarrowThreads, sm, st>>>(a);
+        else mlp_kernel<1, false, kNarrowThreads><<<tiles, kNarrowThreads, sm, st>>>(a);
+    } else if (train) {
         if (mt == 2) mlp_kernel<2, true><<<tiles, kMlpThreads, sm, st>>>(a);
         else mlp_kernel<1, true><<<tiles, kMlpThreads, sm, st>>>(a);
     } else {
