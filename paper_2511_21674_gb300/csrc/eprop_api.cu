@@ -840,7 +840,7 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
         if (persistent || sample_loop) {
             if (i % U != 0) continue;
         } else {
-        eprop::launch_neuron(n, i, (int)net->max_in_per_step, st);
+        eprop::launch_neuron(n, i, (int)net->max_in_per_step, net->sm_count, st);
         fork_readout();
         eprop::launch_readout(n, i, net->sm_count, sr);
         if (n.pred_mode) {
@@ -866,7 +866,7 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
             // after the product: with symmetric feedback B is W_out itself
             fork_readout();
             eprop::launch_readout_weights(n, i, sr);
-            eprop::launch_tables(n, i, st);
+            eprop::launch_tables(n, i, net->sm_count, st);
             L += 4;
             if (c.profile) cudaEventRecordWithFlags(net->ev[2 * nwin], st, cudaEventRecordExternal);
             if (net->trace_mode == 1) {

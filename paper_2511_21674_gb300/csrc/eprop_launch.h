@@ -10,7 +10,7 @@ struct Net;
 struct GridBar;
 
 // neuron updates and input spikes of call step i
-void launch_neuron(const Net &n, int i, int max_events_per_step, cudaStream_t st);
+void launch_neuron(const Net &n, int i, int max_events_per_step, int sm_count, cudaStream_t st);
 void launch_readout(const Net &n, int i, int sm_count, cudaStream_t st);
 // hubs: the hub rows in device memory, null without any
 struct HubRows;
@@ -21,7 +21,7 @@ void prepare_step_kernel_attributes();
 void launch_begin_call(const Net &n, int continuous, cudaStream_t st);
 void launch_end_call(const Net &n, int T, cudaStream_t st);
 void launch_filter_error(const Net &n, int i_end, cudaStream_t st);
-int launch_tables(const Net &n, int i_end, cudaStream_t st);
+int launch_tables(const Net &n, int i_end, int sm_count, cudaStream_t st);
 void launch_trace_window(const Net &n, int i_end, int grid_x, cudaStream_t st);
 // dense window update of a batch (batch > 1 with update windows), one
 // state per sample and synapse

@@ -113,13 +113,18 @@ __device__ __forceinline__ void neuron_update(const Net &n, int i, int b, int j,
 constexpr int kNPT = 2;
 constexpr int kNeuronThreads = 256;
 
-// The first `inject` blocks mark the step's input spikes, the others update
-// neurons.
-// Before its pdl_wait (the predecessor, delivery of the previous step, still
-// runs) a block loads the neurons' state; the ring sums come after it.  At the first step of a call the predecessor may be
-// the kernel that sets the clock, so nothing is read before the wait.
+// opts: the first opts & 0xFFFF blocks mark the step's input spikes, the others
+// update neurons, drawing their drive early or not (in one word: four more bytes
+// of parameters made calls of 20,000 neurons 3 % slower).  Before its pdl_wait (the
+// predecessor, delivery of the previous step, still runs) a block loads the
+// neurons' state and, if early, draws their drive; the ring sums come after it.
+// At the first step of a call the predecessor may be the kernel that sets the
+// clock, so nothing is read before the wait.
+constexpr int kNeuronEarly = 1 << 16;
 template <bool VAR>
-__global__ void __launch_bounds__(kNeuronThreads) neuron_kernel(Net n, int i, int inject) {
+__global__ void __launch_bounds__(kNeuronThreads) neuron_kernel(Net n, int i, int opts) {
+    const int inject = opts & 0xFFFF;
+    const bool early = opts & kNeuronEarly;
     __shared__ uint32_t thr_s[EPROP_MAX_DRIVE_THR];
     __shared__ Clock ck_s;
     __shared__ int len_s;
@@ -152,10 +157,6 @@ __global__ void __launch_bounds__(kNeuronThreads) neuron_kernel(Net n, int i, in
     long long *ring_row = n.ring + ((long long)b * (n.D + 1) + slot) * n.n_rec;
     const long long nb0 = (long long)b * n.n_rec;
     const int jb = (blockIdx.x - inject) * (kNeuronThreads * kNPT) + threadIdx.x;
-    // the drive is drawn before the wait when every block starts early (one
-    // wave: 1e5 neurons 23.2 against 24.1 ms per call), else while the ring loads
-    // are in flight (1e6 neurons 152.7 against 156.4 ms)
-    const bool early = gridDim.x * gridDim.y <= 4 * 152;
     if (i > len) {               // sample already finished: frozen, silent
         pdl_wait();
         pdl_trigger();
@@ -780,7 +781,7 @@ __global__ void __launch_bounds__(kPersThreads) persistent_steps_kernel(Net n, i
 
 // ----------------------------------------------------------------- launches
 
-void launch_neuron(const Net &n, int i, int max_events_per_step, cudaStream_t st) {
+void launch_neuron(const Net &n, int i, int max_events_per_step, int sm_count, cudaStream_t st) {
     const int per_block = kNeuronThreads * kNPT;
     // one group of kNeuronThreads * kNPT neurons per block (a grid capped at
     // the resident blocks, walking several groups per block, measured slower)
@@ -791,10 +792,14 @@ void launch_neuron(const Net &n, int i, int max_events_per_step, cudaStream_t st
         inject = inject < 1 ? 1 : inject > 64 ? 64 : inject;
     }
     const dim3 grid(blocks + inject, n.B);
+    // the drive is drawn before the wait when every block starts early (one wave
+    // of four blocks per SM: 1e5 neurons 23.2 against 24.1 ms per call), else
+    // while the ring loads are in flight (1e6 neurons 152.7 against 156.4 ms)
+    const bool early = (long long)grid.x * grid.y <= 4LL * sm_count;
     if (n.surrogate || n.reset_mode || n.if_period || n.R_win)
-        launch_pdl(neuron_kernel<true>, grid, dim3(kNeuronThreads), 0, st, n, i, inject);
+        launch_pdl(neuron_kernel<true>, grid, dim3(kNeuronThreads), 0, st, n, i, inject | (early ? kNeuronEarly : 0));
     else
-        launch_pdl(neuron_kernel<false>, grid, dim3(kNeuronThreads), 0, st, n, i, inject);
+        launch_pdl(neuron_kernel<false>, grid, dim3(kNeuronThreads), 0, st, n, i, inject | (early ? kNeuronEarly : 0));
 }
 
 void launch_readout(const Net &n, int i, int sm_count, cudaStream_t st) {

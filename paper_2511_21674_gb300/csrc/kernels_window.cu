@@ -1962,11 +1962,11 @@ void launch_filter_error(const Net &n, int i_end, cudaStream_t st) {
     filter_error_kernel<<<tot, 32, 0, st>>>(n);
 }
 
-int launch_tables(const Net &n, int i_end, cudaStream_t st) {
+int launch_tables(const Net &n, int i_end, int sm_count, cudaStream_t st) {
     const bool pair = n.U > 128;         // long LIF windows sweep in FP32 pairs (ALIF always does)
     // blocks of one warp while blocks of four would leave SMs without work
     // (four blocks per SM are resident)
-    const int bd = (long long)n.n_rec * n.B >= 128LL * 4 * 160 ? 128 : 32;
+    const int bd = (long long)n.n_rec * n.B >= 128LL * 4 * sm_count ? 128 : 32;
     const dim3 grid((n.n_rec + bd - 1) / bd, n.B);
 #define EPROP_TAB(A, R, F)                                                                   \
     do {                                                                                     \
