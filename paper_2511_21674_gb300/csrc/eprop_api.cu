@@ -834,7 +834,8 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
     }
     for (int i = 1; i <= T; ++i) {
         if (sample_loop && (i - 1) % U == 0) {
-            eprop::launch_sample_steps(n, i, i + U - 1, st);
+            const cudaError_t le = eprop::launch_sample_steps(n, i, i + U - 1, st);
+            if (le != cudaSuccess && net->launch_err == cudaSuccess) net->launch_err = le;
             L += 1;
         }
         if (persistent || sample_loop) {

@@ -59,7 +59,7 @@ cudaError_t launch_persistent_steps(const Net &n, int T, GridBar *gb, int blocks
 // window) of every sample in one launch
 bool sample_net_small(const Net &n);     // sizes only
 bool sample_steps_fit(const Net &n);     // and the forms the loop serves
-void launch_sample_steps(const Net &n, int i0, int i1, cudaStream_t st);
+cudaError_t launch_sample_steps(const Net &n, int i0, int i1, cudaStream_t st);
 void prepare_sample_attributes();
 void prepare_learning_signal_attributes();
 // band-major learning state (trace_kernel 4)

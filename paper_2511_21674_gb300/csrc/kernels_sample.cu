@@ -543,7 +543,7 @@ bool sample_steps_fit(const Net &n) {
     X(true, 1, 512) X(true, 2, 512) X(true, 4, 512) X(true, 1, 768) X(true, 1, 1024) \
     X(false, 1, 512) X(false, 2, 512) X(false, 4, 512) X(false, 1, 768) X(false, 1, 1024)
 
-void launch_sample_steps(const Net &n, int i0, int i1, cudaStream_t st) {
+cudaError_t launch_sample_steps(const Net &n, int i0, int i1, cudaStream_t st) {
     const SampleShape s = sample_shape(n.n_in, n.n_rec, n.n_out, n.D);
     const size_t sm = sample_smem(s);
     const int nt = s.threads - (s.KR + s.KI) * 32;
@@ -556,10 +556,11 @@ void launch_sample_steps(const Net &n, int i0, int i1, cudaStream_t st) {
 #define EPROP_SMP(V, P, BT)                            \
     if (var == V && npt == P && s.threads == BT) {     \
         sample_steps_kernel<V, P, BT><<<n.B, BT, sm, st>>>(n, i0, i1, lists); \
-        return;                                        \
+        return cudaSuccess;                            \
     }
     EPROP_SMP_EACH(EPROP_SMP)
 #undef EPROP_SMP
+    return cudaErrorInvalidConfiguration;        // a shape without an instance
 }
 
 void prepare_sample_attributes() {

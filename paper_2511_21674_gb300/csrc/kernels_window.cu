@@ -1072,7 +1072,7 @@ __global__ void __launch_bounds__(256, MODE == kPassIdle ? 3 : 2) window_pass_ke
                 if (live[u]) cf[u] = load_coef_dense<ALIF>(n, td[u] & 0xFFFFFFu);
                 if (c0[u] >= 0) t0[u] = load_table<ALIF>(n, qa + (long long)a1 * N + (td[u] & 0xFFFFFFu));
             }
-float G[kB];
+            float G[kB];
 #pragma unroll
             for (int u = 0; u < kB; ++u) {
                 G[u] = 0.f;

@@ -423,8 +423,8 @@ __global__ void refresh_kernel(Layout L, const float *w, long long n) {
 // Adam (Eq. adam1, Eq. adam2, Eq. adam) on the FP32 masters: sums the bias
 // gradients of the row tiles in order, steps, and refreshes the BF16 weights;
 // block 0 also sums the loss.
-__global__ void adam_kernel(Layout L, float *w, float *grad, float *m, float *v, long long n, const float *bpart, const float *lpart, int tiles, float half_inv,
-                            float *loss, float lr, float c1, float c2) {
+__global__ void adam_kernel(Layout L, float *w, float *grad, float *m, float *v, long long n, const float *bpart,
+                            const float *lpart, int tiles, float half_inv, float *loss, float lr, float c1, float c2) {
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
          q += (long long)gridDim.x * blockDim.x) {
         int l;
