@@ -860,7 +860,7 @@ static void issue_call(eprop_net *net, int T, const uint8_t *forced) {
         if (i % U == 0) {
             if (!sample_loop) join_readout();    // nothing forked since the last join otherwise
             fork_readout();
-            eprop::launch_filter_error(n, i, sr);
+            eprop::launch_filter_error(n, i, net->sm_count, sr);
             // L[b][u][j] = sum_k B[j][k] E[b][u][k] of the whole window
             // (Eq. final-gradient), tensor cores with split TF32 operands
             eprop::launch_learning_signals(n.fb, n.E_win, n.L_win, c.n_rec, U, c.n_out, (int)B, n.err_flags, st);

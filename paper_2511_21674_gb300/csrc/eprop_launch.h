@@ -20,7 +20,7 @@ void prepare_kernel_attributes();
 void prepare_step_kernel_attributes();
 void launch_begin_call(const Net &n, int continuous, cudaStream_t st);
 void launch_end_call(const Net &n, int T, cudaStream_t st);
-void launch_filter_error(const Net &n, int i_end, cudaStream_t st);
+void launch_filter_error(const Net &n, int i_end, int sm_count, cudaStream_t st);
 int launch_tables(const Net &n, int i_end, int sm_count, cudaStream_t st);
 void launch_trace_window(const Net &n, int i_end, int grid_x, cudaStream_t st);
 // dense window update of a batch (batch > 1 with update windows), one

@@ -119,6 +119,33 @@ __global__ void __launch_bounds__(32) filter_error_kernel(Net n) {
     if (lane == 0) n.Cwin[idx] = (float)(kap * run);
 }
 
+// The same with one thread per (sample, readout) walking the window: lanes are
+// consecutive readouts, so a 32-byte sector is fetched once, where each of up to
+// eight warps above fetches it for its own readout.  From tens of thousands of
+// (sample, readout) pairs on that traffic costs more than the chain of steps.
+__global__ void __launch_bounds__(128) filter_error_many_kernel(Net n) {
+    const int idx = blockIdx.x * 128 + threadIdx.x;
+    if (idx >= n.B * n.n_out) return;
+    const int b = idx / n.n_out, k = idx % n.n_out, K = n.n_out, U = n.U;
+    const float *__restrict__ E = n.E_win + (long long)b * U * K + k;
+    float *__restrict__ Eb = n.Ebar_win + (long long)b * U * K + k;
+    const double kap = (double)n.kappa + (double)n.kappa_lo;
+    double acc = 0.0;
+    constexpr int kC = 8;
+    for (int u = U; u > 0; u -= kC) {
+        float e[kC];
+#pragma unroll
+        for (int c = 0; c < kC; ++c) e[c] = u - 1 - c >= 0 ? E[(long long)(u - 1 - c) * K] : 0.f;
+#pragma unroll
+        for (int c = 0; c < kC; ++c) {
+            if (u - 1 - c < 0) break;
+            acc = (double)e[c] + kap * acc;
+            Eb[(long long)(u - 1 - c) * K] = (float)acc;
+        }
+    }
+    n.Cwin[idx] = (float)(kap * acc);
+}
+
 // FP32 pairs h + l (|l| about half an ulp of h): about 48 bits.  The products
 // and sums are built from error-free FP32 operations (TwoProduct through the
 // FMA, Knuth's TwoSum; Dekker 1971), spelled out with explicit rounding.
@@ -1956,10 +1983,13 @@ void launch_begin_call(const Net &n, int continuous, cudaStream_t st) {
 
 void launch_end_call(const Net &n, int T, cudaStream_t st) { end_call_kernel<<<1, 32, 0, st>>>(n, T); }
 
-void launch_filter_error(const Net &n, int i_end, cudaStream_t st) {
+void launch_filter_error(const Net &n, int i_end, int sm_count, cudaStream_t st) {
     (void)i_end;
     const int tot = n.B * n.n_out;
-    filter_error_kernel<<<tot, 32, 0, st>>>(n);
+    // a warp / a thread per (sample, readout), windows of 300 steps: 2048 pairs
+    // 18 / 54 us, 8192 59 / 57, 16,384 111 / 58, 65,536 427 / 133
+    if (tot >= 64 * sm_count) filter_error_many_kernel<<<(tot + 127) / 128, 128, 0, st>>>(n);
+    else filter_error_kernel<<<tot, 32, 0, st>>>(n);
 }
 
 int launch_tables(const Net &n, int i_end, int sm_count, cudaStream_t st) {
