@@ -113,18 +113,14 @@ __device__ __forceinline__ void neuron_update(const Net &n, int i, int b, int j,
 constexpr int kNPT = 2;
 constexpr int kNeuronThreads = 256;
 
-// opts: the first opts & 0xFFFF blocks mark the step's input spikes, the others
-// update neurons, drawing their drive early or not (in one word: four more bytes
-// of parameters made calls of 20,000 neurons 3 % slower).  Before its pdl_wait (the
-// predecessor, delivery of the previous step, still runs) a block loads the
-// neurons' state and, if early, draws their drive; the ring sums come after it.
-// At the first step of a call the predecessor may be the kernel that sets the
-// clock, so nothing is read before the wait.
-constexpr int kNeuronEarly = 1 << 16;
+// The first `inject` blocks mark the step's input spikes, the others update
+// neurons.  Before its pdl_wait (the predecessor, delivery of the previous
+// step, still runs) a block loads the neurons' state and, if early, draws their
+// drive; the ring sums come after it.  At the first step of a call the
+// predecessor may be the kernel that sets the clock, so nothing is read before
+// the wait.
 template <bool VAR>
-__global__ void __launch_bounds__(kNeuronThreads) neuron_kernel(Net n, int i, int opts) {
-    const int inject = opts & 0xFFFF;
-    const bool early = opts & kNeuronEarly;
+__global__ void __launch_bounds__(kNeuronThreads) neuron_kernel(Net n, int i, int inject, bool early) {
     __shared__ uint32_t thr_s[EPROP_MAX_DRIVE_THR];
     __shared__ Clock ck_s;
     __shared__ int len_s;
@@ -797,9 +793,9 @@ void launch_neuron(const Net &n, int i, int max_events_per_step, int sm_count, c
     // while the ring loads are in flight (1e6 neurons 152.7 against 156.4 ms)
     const bool early = (long long)grid.x * grid.y <= 4LL * sm_count;
     if (n.surrogate || n.reset_mode || n.if_period || n.R_win)
-        launch_pdl(neuron_kernel<true>, grid, dim3(kNeuronThreads), 0, st, n, i, inject | (early ? kNeuronEarly : 0));
+        launch_pdl(neuron_kernel<true>, grid, dim3(kNeuronThreads), 0, st, n, i, inject, early);
     else
-        launch_pdl(neuron_kernel<false>, grid, dim3(kNeuronThreads), 0, st, n, i, inject | (early ? kNeuronEarly : 0));
+        launch_pdl(neuron_kernel<false>, grid, dim3(kNeuronThreads), 0, st, n, i, inject, early);
 }
 
 void launch_readout(const Net &n, int i, int sm_count, cudaStream_t st) {
