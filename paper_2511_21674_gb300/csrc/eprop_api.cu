@@ -152,6 +152,7 @@ static eprop_status alloc_window(eprop_net *net, int U, int T) {
     if (net->U_alloc == U) return EPROP_OK;
     cudaStreamSynchronize(net->st);
     free_all(net->win_allocs);
+    net->U_alloc = 0;
     if (net->gexec) {
         cudaGraphExecDestroy(net->gexec);
         net->gexec = nullptr;
@@ -656,6 +657,10 @@ extern "C" eprop_status eprop_set_inputs_targets(eprop_net *net, const int64_t *
     } else {
         net->max_in_per_step = 1 << 14;
     }
+    // from here on the earlier inputs are overwritten or their buffers given
+    // back: a call refused below leaves nothing to simulate or read
+    net->have_inputs = 0;
+    net->have_sim = 0;
     // (re)allocate per-T buffers
     if (net->in_allocs.empty() || T != net->T_in || n_in_ids > net->x_cap) {
         cudaStreamSynchronize(net->st);
@@ -685,6 +690,7 @@ extern "C" eprop_status eprop_set_inputs_targets(eprop_net *net, const int64_t *
         if (net->pred && (n.pred_mode & 2)) IA(pred_rec, float, B * T * n.pred_in);
 #undef IA
         net->x_cap = cap;
+        net->T_in = T;                  // the buffers' size, also if the call is refused below
     }
     n.T = T;
     cudaStream_t st = net->st;
