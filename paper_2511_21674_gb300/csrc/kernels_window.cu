@@ -1195,7 +1195,7 @@ __global__ void __launch_bounds__(256, MODE == kPassIdle ? 3 : 2) window_pass_ke
 // conversion and an addition of 16 cycles per warp each (2 FP64 lanes per
 // SM).  Lanes of a warp read consecutive targets of one (sample, step).
 // Measured (batch 64, 2512 rows, 5e7 arrivals): one warp per row with FP64
-// sums and a four-float table 705 us; this form 94 us; batch 32 of 2200
+// sums and a four-float table 705 us; this form 89 us; batch 32 of 2200
 // steps, 140 rows: 2063 -> 74 us.
 // A pair that has left FP32's range (or met an infinity: inf - inf is NaN) is
 // formed again in FP64 from the spike bits.
@@ -1367,7 +1367,7 @@ __global__ void __launch_bounds__(kTbThreads, kTbBlocks) trace_batched_kernel(Ne
 // sum do not change), so that 64 finite ones cannot leave FP32's range, where
 // the addition's error would be inf - inf; a check per addition cost 2 % of a
 // call.  Measured (batch 64, 2512 rows, 4.7e5 synapses, windows of 50 steps,
-// FP32 traces): one warp per row, FP64 sums 452 us per window; this form 193 us.
+// FP32 traces): one warp per row, FP64 sums 452 us per window; this form 198 us.
 //
 // R: rows of a group.  The block is one group of four rows, or, where rows are
 // many and short (row_per_warp), eight groups (a warp each) of one row: a block
